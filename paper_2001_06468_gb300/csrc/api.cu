@@ -84,6 +84,7 @@ nrs_status alloc_all(Ctx *c)
         {(void **)&c->d_gj_cb, sizeof(float) * 4 * 64 * lda},
         {(void **)&c->d_gj_stage, sizeof(float) * 4 * 64 * 64},
         {(void **)&c->d_gj_sync, sizeof(int32_t) * 4},
+        {(void **)&c->d_asm_claim, sizeof(unsigned int)},
         {(void **)&c->d_info, sizeof(int32_t)},
         {(void **)&c->d_r, sizeof(double) * lda},
         {(void **)&c->d_w, sizeof(double) * lda},
@@ -138,7 +139,7 @@ void free_all(Ctx *c)
                     c->d_gj_rt,  c->d_gj_cb,  c->d_dpart,  c->d_bar,        c->d_pg_stats,
                     c->d_step_stats, c->d_Xsh, c->d_Xsl, c->d_xh, c->d_xl, c->d_gj_stage, c->d_gj_sync, c->d_part32,
                     c->d_part_fx, c->d_vf, c->d_gj2, c->d_gj2_r,
-                    c->d_vf2, c->d_Adf};
+                    c->d_vf2, c->d_Adf, c->d_asm_claim};
     for (void *p : ptrs)
         if (p) cudaFree(p);
     void *tr[] = {c->d_tr, c->d_tr_save, c->d_tr_u, c->d_tr_part, c->d_vel_part, c->d_dp_K,
@@ -229,8 +230,10 @@ nrs_status do_factor(Ctx *c, int prec)
 
 // write_lo: also write the FP32 copy (which a Gauss-Jordan factor replaces by
 // its inverse: writing it destroys that factor).
+// wait64: the caller's next work needs the FP64 matrix, so its assembly takes
+// the whole GPU instead of the side stream.
 nrs_status do_segments_and_assemble(Ctx *c, const D4 *x_lab, const D4 *Xw_lab, bool write_lo = true,
-                                    bool from_state = false)
+                                    bool from_state = false, bool wait64 = false)
 {
     nrs::launch_gather(*c, Xw_lab, c->d_seg_ptr, c->d_perm);
     float *a32 = (c->factor_prec == NRS_FP64 || !write_lo) ? nullptr : c->d_A32;
@@ -241,11 +244,15 @@ nrs_status do_segments_and_assemble(Ctx *c, const D4 *x_lab, const D4 *Xw_lab, b
         // then the FP64 matrix on the side stream beside the factorisation,
         // joined before the refinement uses it
         nrs::launch_assemble32(*c, x_lab, a32, c->lda);
-        CK(cudaEventRecord(c->ev_asm, c->stream));
-        CK(cudaStreamWaitEvent(c->stream3, c->ev_asm, 0));
-        nrs::launch_assemble(*c, x_lab, c->d_A64, nullptr, c->lda, c->stream3, from_state);
-        CK(cudaEventRecord(c->ev_asm_done, c->stream3));
-        c->asm_pending = true;
+        if (wait64) {
+            nrs::launch_assemble(*c, x_lab, c->d_A64, nullptr, c->lda, nullptr, from_state);
+        } else {
+            CK(cudaEventRecord(c->ev_asm, c->stream));
+            CK(cudaStreamWaitEvent(c->stream3, c->ev_asm, 0));
+            nrs::launch_assemble(*c, x_lab, c->d_A64, nullptr, c->lda, c->stream3, from_state);
+            CK(cudaEventRecord(c->ev_asm_done, c->stream3));
+            c->asm_pending = true;
+        }
     } else {
         // one FP64 pass; with an FP32 copy, that copy is the rounded FP64 entries
         nrs::launch_assemble(*c, x_lab, c->d_A64, a32, c->lda, nullptr, from_state);
@@ -769,10 +776,10 @@ nrs_status nrs_assemble(nrs_ctx *ctx, const double *x, const double *Xw, double 
     if (!c || !x || !Xw) return fail(c, NRS_EINVAL, "nrs_assemble: null argument");
     if (!c->seg_valid) return fail(c, NRS_EINVAL, "nrs_assemble before nrs_nearest_build");
     if (A64 && lda < c->n) return fail(c, NRS_EINVAL, "nrs_assemble: lda < n");
-    nrs_status st = do_segments_and_assemble(c, (const D4 *)x, (const D4 *)Xw);
+    nrs_status st = do_segments_and_assemble(c, (const D4 *)x, (const D4 *)Xw, true, false,
+                                             A64 != nullptr);
     if (st != NRS_OK) return st;
     if (A64) {
-        nrs::join_assembly(*c);
         CK(cudaMemcpy2DAsync(A64, sizeof(double) * lda, c->d_A64, sizeof(double) * c->lda,
                              sizeof(double) * c->n, c->n, cudaMemcpyDeviceToDevice, c->stream));
     }

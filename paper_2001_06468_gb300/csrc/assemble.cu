@@ -22,6 +22,7 @@
 
 #include <algorithm>
 
+#include "fp64_int.cuh"
 #include "nrs_internal.cuh"
 
 namespace nrs {
@@ -30,14 +31,57 @@ constexpr int AS_THREADS = (int)kAssembleTileM;
 constexpr int AS_NT = (int)kAssembleTileN;
 constexpr int AS_CHUNK = 512;
 // the FP64 kernel runs beside the fused factorisation, whose CTA takes about
-// 195 KB of an SM's shared memory: its staging chunk is kept at 8 KB so that
+// 195 KB of an SM's shared memory: its staging chunk is kept at 6 KB so that
 // up to three of its CTAs still fit beside one (the order of the sums over q
 // does not depend on the chunk)
-constexpr int AS64_CHUNK = 256;
+constexpr int AS64_CHUNK = 128;
 
 struct Acc6 {
     double xx, xy, xz, yy, yz, zz;
 };
+
+// FP64 additions and products as fused multiply-adds: GB300 issues an FP64
+// fused multiply-add every 64 clocks per scheduler, a plain add or multiply
+// every 76.  `one` is 1.0 and `nz` is -0.0, passed at run time so that the
+// compiler does not turn them back; a 1 + b and a b + (-0.0) round exactly as
+// a + b and a b do (signed zeros included).
+struct FmaOps {
+    double one, nz;
+    __device__ __forceinline__ double add(double a, double b) const { return __fma_rn(a, one, b); }
+    __device__ __forceinline__ double sub(double a, double b) const { return __fma_rn(b, -one, a); }
+    __device__ __forceinline__ double mul(double a, double b) const { return __fma_rn(a, b, nz); }
+};
+
+// A quadrature point staged for the pair loop: its weight also as a
+// significand for the integer products (shifted left by one, sign and
+// exponent field), usable when `ok`.
+struct alignas(16) StagedX {
+    double x, y, z, w;
+    uint64_t w2;
+    uint32_t wf, ok;
+};
+
+__device__ __forceinline__ StagedX stage_point(const D4 &p)
+{
+    StagedX v;
+    v.x = p.x;
+    v.y = p.y;
+    v.z = p.z;
+    v.w = p.w;
+    const Sig sw = unpack(p.w);
+    v.w2 = sw.m << 1;
+    v.wf = sw.f;
+    // 2^-200 <= |w| < 2^200 (zero, subnormal and non-finite weights excluded)
+    const uint32_t ex = (sw.f >> 20) & 0x7ffu;
+    v.ok = ex - 823u < 400u;
+    return v;
+}
+
+__device__ __forceinline__ float2 df_split_int(double v)
+{
+    float hi, lo;
+    return split_pair(v, hi, lo) ? make_float2(hi, lo) : df_split(v);
+}
 
 // The FP64 entries are the definition evaluated term by term in one fixed
 // order, with every operation rounded on its own (no fused multiply-add,
@@ -48,62 +92,183 @@ struct Acc6 {
 // so each entry is a deterministic function of the inputs, independent of
 // the tiling and of the device.
 __device__ __forceinline__ void flush_block(int64_t m, int64_t n, const Acc6 &a, double c,
-                                            double *__restrict__ A64, float *__restrict__ A32,
-                                            float2 *__restrict__ Adf, int64_t lda)
+                                            const FmaOps &op, double *__restrict__ A64,
+                                            float *__restrict__ A32, float2 *__restrict__ Adf,
+                                            int64_t lda)
 {
-    const double v[9] = {__dmul_rn(a.xx, c), __dmul_rn(a.xy, c), __dmul_rn(a.xz, c),
-                         __dmul_rn(a.xy, c), __dmul_rn(a.yy, c), __dmul_rn(a.yz, c),
-                         __dmul_rn(a.xz, c), __dmul_rn(a.yz, c), __dmul_rn(a.zz, c)};
+    const double v[6] = {op.mul(a.xx, c), op.mul(a.xy, c), op.mul(a.xz, c),
+                         op.mul(a.yy, c), op.mul(a.yz, c), op.mul(a.zz, c)};
+    constexpr int at[9] = {0, 1, 2, 1, 3, 4, 2, 4, 5};
+    const int64_t col = 3 * n * lda + 3 * m;
 #pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        const int64_t col = (3 * n + k) * lda + 3 * m;
+    for (int k = 0; k < 3; ++k)
 #pragma unroll
-        for (int j = 0; j < 3; ++j) {
-            A64[col + j] = v[3 * j + k];
-            if (A32) A32[col + j] = (float)v[3 * j + k];
-            if (Adf) Adf[col + j] = df_split(v[3 * j + k]);
-        }
+        for (int j = 0; j < 3; ++j) A64[col + k * lda + j] = v[at[3 * j + k]];
+    if (A32) {
+#pragma unroll
+        for (int k = 0; k < 3; ++k)
+#pragma unroll
+            for (int j = 0; j < 3; ++j) A32[col + k * lda + j] = (float)v[at[3 * j + k]];
+    }
+    if (Adf) {
+        float2 f[6];
+#pragma unroll
+        for (int i = 0; i < 6; ++i) f[i] = df_split_int(v[i]);
+#pragma unroll
+        for (int k = 0; k < 3; ++k)
+#pragma unroll
+            for (int j = 0; j < 3; ++j) Adf[col + k * lda + j] = f[at[3 * j + k]];
     }
 }
 
-__device__ __forceinline__ void add_pair(double mx, double my, double mz, const D4 &X,
-                                         double eps2, double two_e2, Acc6 &a)
+// The six terms S_jk w on the FP64 pipe: the general path, for the pairs whose
+// operands leave the integer path's range (zero or extreme weights, distances
+// beyond 2^50 or below 2^-50, non-finite values) or meet a rounding tie there.
+__device__ __forceinline__ Acc6 terms_fp64(double mx, double my, double mz, const StagedX &X,
+                                           double eps2, double two_e2)
 {
     const double rx = __dsub_rn(mx, X.x), ry = __dsub_rn(my, X.y), rz = __dsub_rn(mz, X.z);
     const double r2 = __dadd_rn(__dadd_rn(__dmul_rn(rx, rx), __dmul_rn(ry, ry)), __dmul_rn(rz, rz));
     const double rho = __dadd_rn(r2, eps2);
     const double s = __ddiv_rn(1.0, __dmul_rn(rho, __dsqrt_rn(rho)));
-    const double dg = __dadd_rn(r2, two_e2);
-    const double w = X.w;
-    a.xx = __dadd_rn(a.xx, __dmul_rn(__dmul_rn(__dadd_rn(__dmul_rn(rx, rx), dg), s), w));
-    a.xy = __dadd_rn(a.xy, __dmul_rn(__dmul_rn(__dmul_rn(rx, ry), s), w));
-    a.xz = __dadd_rn(a.xz, __dmul_rn(__dmul_rn(__dmul_rn(rx, rz), s), w));
-    a.yy = __dadd_rn(a.yy, __dmul_rn(__dmul_rn(__dadd_rn(__dmul_rn(ry, ry), dg), s), w));
-    a.yz = __dadd_rn(a.yz, __dmul_rn(__dmul_rn(__dmul_rn(ry, rz), s), w));
-    a.zz = __dadd_rn(a.zz, __dmul_rn(__dmul_rn(__dadd_rn(__dmul_rn(rz, rz), dg), s), w));
+    const double dg = __dadd_rn(r2, two_e2), w = X.w;
+    Acc6 v;
+    v.xx = __dmul_rn(__dmul_rn(__dadd_rn(__dmul_rn(rx, rx), dg), s), w);
+    v.xy = __dmul_rn(__dmul_rn(__dmul_rn(rx, ry), s), w);
+    v.xz = __dmul_rn(__dmul_rn(__dmul_rn(rx, rz), s), w);
+    v.yy = __dmul_rn(__dmul_rn(__dadd_rn(__dmul_rn(ry, ry), dg), s), w);
+    v.yz = __dmul_rn(__dmul_rn(__dmul_rn(ry, rz), s), w);
+    v.zz = __dmul_rn(__dmul_rn(__dadd_rn(__dmul_rn(rz, rz), dg), s), w);
+    return v;
 }
 
-// One tile = AS_THREADS collocation points x AS_NT segments; tiles are taken
-// in grid-stride order (tile = mx + gx * ny), so the kernel also runs on a
-// capped grid beside the factorisation.
-__global__ void __launch_bounds__(AS_THREADS)
+// Squared distances below this component count as zero in terms_int.
+constexpr uint32_t kTinyHi = 873u << 20;  // 2^-150
+
+__device__ __forceinline__ bool tiny(double r)
+{
+    return (hi32(double_bits(r)) & 0x7fffffffu) < kTinyHi;
+}
+
+// The terms of one pair, without a branch.  The FP64 pipe bounds this kernel,
+// so it is left the 16 additions and subtractions; the square root, the
+// reciprocal and the 18 products r_j r_k, s and w run beside it on the integer
+// pipe, rounded identically (fp64_int.cuh).  A component of r below 2^-150 is
+// taken as zero (then a product with it is a zero, whose sign does not matter:
+// a sum starts at +0).  odd = 1: some component was; 2 and more: the general
+// path is needed.
+__device__ __forceinline__ Acc6 terms_int(double mx, double my, double mz, const StagedX &X,
+                                          double eps2, double two_e2, const FmaOps &op, int &odd)
+{
+    const double rx = op.sub(mx, X.x), ry = op.sub(my, X.y), rz = op.sub(mz, X.z);
+    const bool tx = tiny(rx), ty = tiny(ry), tz = tiny(rz);
+    const Sig ux = unpack(rx), uy = unpack(ry), uz = unpack(rz);
+    bool bad = !X.ok;
+    const Sig pxx = mul_sig(ux, ux.m << 1, ux.f, bad);
+    const Sig pyy = mul_sig(uy, uy.m << 1, uy.f, bad);
+    const Sig pzz = mul_sig(uz, uz.m << 1, uz.f, bad);
+    const double xx = tx ? 0.0 : pack(pxx), yy = ty ? 0.0 : pack(pyy), zz = tz ? 0.0 : pack(pzz);
+    const double r2 = op.add(op.add(xx, yy), zz);
+    const double rho = op.add(r2, eps2);
+    const double dg = op.add(r2, two_e2);
+    // rho in [2^-100, 2^100)
+    bad |= (hi32(double_bits(rho)) - (923u << 20)) >= (200u << 20);
+    const Sig s = inv_rho_sqrt(rho, bad);
+    const uint64_t s2 = s.m << 1;
+    auto term = [&](const Sig &p) {
+        return pack(mul_sig(mul_sig(p, s2, s.f, bad), X.w2, X.wf, bad));
+    };
+    Acc6 v;
+    v.xx = term(unpack(op.add(xx, dg)));
+    v.yy = term(unpack(op.add(yy, dg)));
+    v.zz = term(unpack(op.add(zz, dg)));
+    const double xy = term(mul_sig(ux, uy.m << 1, uy.f, bad));
+    const double xz = term(mul_sig(ux, uz.m << 1, uz.f, bad));
+    const double yz = term(mul_sig(uy, uz.m << 1, uz.f, bad));
+    v.xy = tx || ty ? 0.0 : xy;
+    v.xz = tx || tz ? 0.0 : xz;
+    v.yz = ty || tz ? 0.0 : yz;
+    odd = (bad ? 2 : 0) | (tx || ty || tz ? 1 : 0);
+    return v;
+}
+
+__device__ __noinline__ Acc6 terms_fp64_call(double mx, double my, double mz, const StagedX *X,
+                                             double eps2, double two_e2)
+{
+    return terms_fp64(mx, my, mz, *X, eps2, two_e2);
+}
+
+// terms_int's pairs with odd != 0: components taken as zero must be zero (the
+// coordinates the same bits); anything else takes the general path.
+__device__ __forceinline__ void settle(double mx, double my, double mz, const StagedX &X,
+                                       double eps2, double two_e2, const FmaOps &op, int odd,
+                                       Acc6 &v)
+{
+    if (odd == 0) return;
+    if (odd == 1) {
+        const double a[3] = {mx, my, mz}, b[3] = {X.x, X.y, X.z};
+#pragma unroll
+        for (int i = 0; i < 3; ++i)
+            if (double_bits(a[i]) != double_bits(b[i]) && tiny(op.sub(a[i], b[i]))) odd = 2;
+    }
+    if (odd >= 2) v = terms_fp64_call(mx, my, mz, &X, eps2, two_e2);
+}
+
+__device__ __forceinline__ void add_terms(const FmaOps &op, const Acc6 &v, Acc6 &a)
+{
+    a.xx = op.add(a.xx, v.xx);
+    a.xy = op.add(a.xy, v.xy);
+    a.xz = op.add(a.xz, v.xz);
+    a.yy = op.add(a.yy, v.yy);
+    a.yz = op.add(a.yz, v.yz);
+    a.zz = op.add(a.zz, v.zz);
+}
+
+// What bounds it: the FP64 pipe (INT: 16 additions a pair at 64 clocks a warp
+// and scheduler, 1024 of about 1150 clocks), with the integer pipe nearly as
+// busy.  4680 force and 37440 quadrature points, with the float-pair copy:
+// 17.2 ms with all of a pair's operations on the FP64 pipe (about 3580
+// clocks), 7.9 ms with the products with s and w, the square root and the
+// reciprocal on the integer pipe, 5.3 ms with the products r_j r_k there too.
+// Two quadrature points at a time were slower (128 registers); 96 registers
+// (five CTAs an SM) measured best of 80, 96 and 114.
+//
+// One tile = AS_THREADS collocation points x NT segments (NT a power of two,
+// at most AS_NT), tile = mx + gx * ny.  A full grid takes one tile per CTA.
+// Beside the factorisation (`claim` given: a counter that starts at zero) the
+// grid is capped and its CTAs claim tiles one at a time: where other kernels'
+// CTAs share an SM, or the scheduler put more of these CTAs on it, they take
+// fewer. 
+template <bool INT>
+__global__ void __launch_bounds__(AS_THREADS, INT ? 5 : 8)
     k_assemble64(int64_t N, const D4 *__restrict__ x, const D4 *__restrict__ Xs,
-                 const int32_t *__restrict__ seg_ptr, double eps2, double c,
+                 const int32_t *__restrict__ seg_ptr, double eps2, double c, FmaOps op,
                  double *__restrict__ A64, float *__restrict__ A32, float2 *__restrict__ Adf,
-                 int64_t lda, int64_t gx,
-                 int64_t tiles, const uint8_t *__restrict__ mblk_keep,
+                 int64_t lda, int64_t gx, int NT,
+                 int64_t tiles, unsigned int *claim, const uint8_t *__restrict__ mblk_keep,
                  const uint8_t *__restrict__ nblk_keep)
 {
-    __shared__ D4 sX[AS64_CHUNK];
+    __shared__ StagedX sX[AS64_CHUNK];
     __shared__ int32_t sp[AS_NT + 1];
-    for (int64_t tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+    __shared__ unsigned int s_tile;
+    for (;;) {
+    int64_t tile = blockIdx.x;
+    if (claim) {
+        if (threadIdx.x == 0) s_tile = atomicAdd(claim, 1u);
+        __syncthreads();
+        tile = s_tile;
+    }
+    if (tile >= tiles) return;
+    const int64_t n0 = (tile / gx) * NT;
     // a tile whose collocation points and segments all belong to static rigid
     // bodies keeps the entries of the previous assembly (the same values)
-    if (mblk_keep && mblk_keep[tile % gx] && nblk_keep[tile / gx]) continue;
-    __syncthreads();  // the previous tile is done with sp and sX
+    if (mblk_keep && mblk_keep[tile % gx] && nblk_keep[n0 / AS_NT]) {
+        if (!claim) return;
+        __syncthreads();  // everyone has read s_tile
+        continue;
+    }
     const int64_t m = (tile % gx) * AS_THREADS + threadIdx.x;
-    const int64_t n0 = (tile / gx) * AS_NT;
-    const int nt = (int)min((int64_t)AS_NT, N - n0);
+    const int nt = (int)min((int64_t)NT, N - n0);
     if (threadIdx.x <= nt) sp[threadIdx.x] = seg_ptr[n0 + threadIdx.x];
     const bool active = m < N;
     double mx = 0.0, my = 0.0, mz = 0.0;
@@ -122,24 +287,37 @@ __global__ void __launch_bounds__(AS_THREADS)
         const int cnt = min(AS64_CHUNK, qend - c0);
         const int32_t cend = c0 + cnt;
         __syncthreads();
-        for (int i = threadIdx.x; i < cnt; i += AS_THREADS) sX[i] = Xs[c0 + i];
+        for (int i = threadIdx.x; i < cnt; i += AS_THREADS) sX[i] = stage_point(Xs[c0 + i]);
         __syncthreads();
         // segment by segment (bounds uniform across the block): the sums run
         // in ascending q within each segment
         while (cur < nt) {
             const int32_t sb = max(sp[cur], c0), se = min(sp[cur + 1], cend);
-            for (int32_t q = sb; q < se; ++q) add_pair(mx, my, mz, sX[q - c0], eps2, two_e2, a);
+            for (int32_t q = sb; q < se; ++q) {
+                const StagedX &X = sX[q - c0];
+                Acc6 v;
+                if (INT) {
+                    int odd;
+                    v = terms_int(mx, my, mz, X, eps2, two_e2, op, odd);
+                    settle(mx, my, mz, X, eps2, two_e2, op, odd, v);
+                } else {
+                    v = terms_fp64(mx, my, mz, X, eps2, two_e2);
+                }
+                add_terms(op, v, a);
+            }
             if (sp[cur + 1] > cend) break;  // the segment continues in the next chunk
-            if (active) flush_block(m, n0 + cur, a, c, A64, A32, Adf, lda);
+            if (active) flush_block(m, n0 + cur, a, c, op, A64, A32, Adf, lda);
             a = Acc6{0, 0, 0, 0, 0, 0};
             ++cur;
         }
     }
     while (cur < nt) {
-        if (active) flush_block(m, n0 + cur, a, c, A64, A32, Adf, lda);
+        if (active) flush_block(m, n0 + cur, a, c, op, A64, A32, Adf, lda);
         a = Acc6{0, 0, 0, 0, 0, 0};
         ++cur;
     }
+    if (!claim) return;
+    __syncthreads();  // everyone is done with s_tile, sp and sX
     }  // tile loop
 }
 
@@ -147,9 +325,10 @@ __global__ void __launch_bounds__(AS_THREADS)
 // lo = (float)(p - hi), so that differences of nearby points are formed in
 // FP32 without losing the digits that the FP64 difference keeps.
 __global__ void k_split_points(int64_t count, const D4 *__restrict__ p, float4 *__restrict__ hi,
-                               float4 *__restrict__ lo)
+                               float4 *__restrict__ lo, unsigned int *claim)
 {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i == 0) *claim = 0;
     if (i >= count) return;
     const D4 v = p[i];
     const float hx = (float)v.x, hy = (float)v.y, hz = (float)v.z;
@@ -359,30 +538,45 @@ void launch_assemble(Ctx &c, const D4 *x_lab, double *A64, float *A32, int64_t l
     if (!attr) {
         // beside the factorisation, whose diagonal inverse needs a large
         // shared-memory carveout on the SM it lands on
-        cudaFuncSetAttribute(k_assemble64, cudaFuncAttributePreferredSharedMemoryCarveout,
-                             cudaSharedmemCarveoutMaxShared);
+        for (auto k : {k_assemble64<true>, k_assemble64<false>})
+            cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                 cudaSharedmemCarveoutMaxShared);
         attr = true;
     }
-    const int64_t gx = ceil_div(c.N, AS_THREADS), tiles = gx * ceil_div(c.N, AS_NT);
-    // beside the factorisation: a few CTAs of four warps per SM (about 25 KB of
-    // shared memory and 24K registers), grid-stride over the tiles, so the
-    // factorisation's kernels (one CTA per SM each) still find room on every SM
-    const int64_t grid = side ? std::min<int64_t>(tiles, (int64_t)c.asm_side_ctas * c.num_sms)
-                              : tiles;
+    // segments of a tile: AS_NT, halved while there are too few tiles to fill
+    // and balance the SMs (a tile's segments are summed one after the other)
+    const int64_t gx = ceil_div(c.N, AS_THREADS);
+    int nt = AS_NT;
+    while (nt > 1 && gx * ceil_div(c.N, nt) < 16 * (int64_t)c.num_sms) nt /= 2;
+    const int64_t tiles = gx * ceil_div(c.N, nt);
     const double coef = 1.0 / (8.0 * kPi * c.mu);
+    const FmaOps op{1.0, -0.0};
+    float2 *df = (c.arnoldi_df && A64 == c.d_A64) ? c.d_Adf : nullptr;
     c.tbeg(PH_ASSEMBLE, s);
     // the blocks among static rigid bodies do not change from one state to the
     // next: kept in the context's FP64 matrix once it holds them (only for an
     // FP64-only pass over the context's own state)
     const bool keep = from_state && A32 == nullptr && A64 == c.d_A64 && c.have_static &&
                       c.static_cache_valid;
-    k_assemble64<<<(unsigned)grid, AS_THREADS, 0, s>>>(c.N, x_lab, c.d_Xs, c.d_seg_ptr,
-                                                       c.eps * c.eps, coef, A64, A32,
-                                                       (c.arnoldi_df && A64 == c.d_A64) ? c.d_Adf
-                                                                                        : nullptr,
-                                                       lda, gx,
-                                                       tiles, keep ? c.d_mblk_keep : nullptr,
-                                                       keep ? c.d_nblk_keep : nullptr);
+    const uint8_t *mkeep = keep ? c.d_mblk_keep : nullptr, *nkeep = keep ? c.d_nblk_keep : nullptr;
+    int64_t grid = tiles;
+    auto kernel = k_assemble64<true>;
+    if (side) {
+        // beside the factorisation: a few CTAs of four warps per SM, claiming
+        // tiles, so that the factorisation's kernels (one CTA per SM each) still
+        // find room on every SM.  A lone one-level factorisation outlasts the
+        // assembly either way, and its chain of latency-bound kernels suffers
+        // more from the integer form's issue slots and registers than from the
+        // FP64 form's longer run (single swimmer's step: 3.18 ms with the FP64
+        // form, 3.27 with the integer one); among the chains of a batch (32
+        // reduced nodes: 37.1 and 25.2 ms) and beside the two-level updates the
+        // integer form is the better one.
+        if (!c.pg_shared && c.n < GJ2_MIN_N) kernel = k_assemble64<false>;
+        grid = std::min<int64_t>(tiles, (int64_t)c.asm_side_ctas * c.num_sms);
+    }
+    kernel<<<(unsigned)grid, AS_THREADS, 0, s>>>(
+        c.N, x_lab, c.d_Xs, c.d_seg_ptr, c.eps * c.eps, coef, op, A64, A32, df, lda, gx, nt, tiles,
+        side ? c.d_asm_claim : nullptr, mkeep, nkeep);
     c.static_cache_valid = from_state && A64 == c.d_A64;
     c.tend(PH_ASSEMBLE, s);
     c.launches += 1;
@@ -393,8 +587,10 @@ void launch_assemble32(Ctx &c, const D4 *x_lab, float *A32, int64_t lda)
     dim3 grid((unsigned)ceil_div(c.N, AS32_M), (unsigned)ceil_div(c.N, AS_NT));
     const float coef = (float)(1.0 / (8.0 * kPi * c.mu));
     c.tbeg(PH_ASSEMBLE32);
-    k_split_points<<<(unsigned)ceil_div(c.N, 256), 256, 0, c.stream>>>(c.N, x_lab, c.d_xh, c.d_xl);
-    k_split_points<<<(unsigned)ceil_div(c.Q, 256), 256, 0, c.stream>>>(c.Q, c.d_Xs, c.d_Xsh, c.d_Xsl);
+    k_split_points<<<(unsigned)ceil_div(c.N, 256), 256, 0, c.stream>>>(c.N, x_lab, c.d_xh, c.d_xl,
+                                                                            c.d_asm_claim);
+    k_split_points<<<(unsigned)ceil_div(c.Q, 256), 256, 0, c.stream>>>(c.Q, c.d_Xs, c.d_Xsh, c.d_Xsl,
+                                                                            c.d_asm_claim);
     k_assemble32<<<grid, AS_THREADS, 0, c.stream>>>(c.N, c.d_xh, c.d_xl, c.d_Xsh, c.d_Xsl,
                                                     c.d_seg_ptr, (float)(c.eps * c.eps), coef, A32,
                                                     lda);

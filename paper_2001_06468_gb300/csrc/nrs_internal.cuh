@@ -169,6 +169,7 @@ struct Ctx {
     bool asm_pending = false;                    // stream3 holds an FP64 assembly not yet joined
     int lo_eval = 0;  // FP32 copy for the factor: 0 evaluated in FP32 (overlapped), 1 rounded FP64
     int asm_side_ctas = 3;  // CTAs per SM of the FP64 assembly beside the factorisation
+    unsigned int *d_asm_claim = nullptr;  // its tile counter there
     cudaEvent_t ev_upd = nullptr, ev_diag = nullptr;
     cudaStream_t stream4 = nullptr;              // finish step of the factorisation
     cudaEvent_t ev_fin_ready = nullptr, ev_fin[2] = {nullptr, nullptr};

@@ -424,7 +424,7 @@ nrs_status nrs_get_tracers(nrs_ctx *ctx, double *xp);
  *
  * No context, no cudaMalloc/cudaFree, no allocating library call.  The
  * caller passes the inputs and outputs; the scratch (segment counters, the
- * block task table, the body offsets, a status word; about 0.4 MB) lives in
+ * block task table, the body offsets, the force points' boxes, a status word; about 0.5 MB) lives in
  * file-scope device arrays of fixed size that every GPU loading the library
  * holds until the process exits.
  *   x [N*4], Xw [Q*4]      device, as for nrs_nearest_build (body frame for

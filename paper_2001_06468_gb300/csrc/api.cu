@@ -69,6 +69,7 @@ nrs_status alloc_all(Ctx *c)
         {(void **)&c->d_b, sizeof(double) * lda},
         {(void **)&c->d_sol, sizeof(double) * 2 * lda},
         {(void **)&c->d_nn, sizeof(int32_t) * Q},
+        {(void **)&c->d_nn_box, 2 * sizeof(float4) * nrs::ceil_div(N, nrs::NN_BOX)},
         {(void **)&c->d_seg_ptr, sizeof(int32_t) * (N + 1)},
         {(void **)&c->d_perm, sizeof(int32_t) * Q},
         {(void **)&c->d_cursor, sizeof(int32_t) * (N + 1)},
@@ -139,7 +140,7 @@ void free_all(Ctx *c)
                     c->d_gj_rt,  c->d_gj_cb,  c->d_dpart,  c->d_bar,        c->d_pg_stats,
                     c->d_step_stats, c->d_Xsh, c->d_Xsl, c->d_xh, c->d_xl, c->d_gj_stage, c->d_gj_sync, c->d_part32,
                     c->d_part_fx, c->d_vf, c->d_gj2, c->d_gj2_r,
-                    c->d_vf2, c->d_Adf, c->d_asm_claim};
+                    c->d_vf2, c->d_Adf, c->d_asm_claim, c->d_nn_box};
     for (void *p : ptrs)
         if (p) cudaFree(p);
     void *tr[] = {c->d_tr, c->d_tr_save, c->d_tr_u, c->d_tr_part, c->d_vel_part, c->d_dp_K,

@@ -3,6 +3,7 @@
 // and Sec. 4).
 #include <math.h>
 
+#include "fp64_int.cuh"
 #include "nrs_internal.cuh"
 
 namespace nrs {
@@ -96,7 +97,20 @@ void launch_kinematics(Ctx &c, const D4 *xi, const D4 *Xiw, const D4 *xidot, D4 
 // nearest neighbours (Sec. 3: n-hat(q) = argmin_n |x[n] - X[q]|)
 // ---------------------------------------------------------------------------
 //
-// Two passes over the candidate force points, staged through shared memory.
+// The force points are boxed 32 at a time (k_nn_boxes), and a warp only looks
+// at the boxes that can hold a nearest neighbour of one of its 8 quadrature
+// points: it evaluates the box whose centre is closest to that of its own
+// points' box, which bounds every point's distance from above, and keeps the
+// boxes whose distance from its own box does not exceed the largest of these
+// bounds.  The block stages the boxes that any of its warps kept, each warp
+// scans its own.  Points that are neighbours in index order are neighbours in
+// space on lattices and curves, so few boxes remain; for points in arbitrary
+// order all do, and the scan is the full one.  9200 force points and 92000
+// quadrature points of the channel, over all bodies: 893 us for the scan of
+// all pairs, 270 us with boxes kept for a whole block (those that straddle
+// two faces keep nearly all), 129 us kept by warps.
+//
+// Two passes over the kept force points, staged through shared memory.
 // Pass 1 finds m_f, the smallest FP32 squared distance.  With C the largest
 // coordinate magnitude involved, every FP32 difference component is within
 // delta = 2^-24 (|x| + |X| + |dx|) <= 4.01 * 2^-24 * C of the exact one, so
@@ -108,8 +122,63 @@ void launch_kinematics(Ctx &c, const D4 *xi, const D4 *Xiw, const D4 *xidot, D4 
 // ((dx*dx + dy*dy) + dz*dz), keeping the first strict minimum in ascending
 // index order.  The 1e-6 factors dominate every FP32 rounding of the bound
 // itself (u = 2^-24 ~ 6e-8), so the result equals an exhaustive FP64 search.
+// The same bound on a distance from above, taken over the warp, is compared
+// with the boxes' squared distances from below: the boxes are rounded outward,
+// and the FP32 rounding of the distance between two boxes (relative, 6 u) is
+// again inside the 1e-6 factors.
 
-constexpr int NN_TILE = 512;
+constexpr int NN_TILE = 512;                       // force points staged at a time
+constexpr int NN_BOXES = NN_TILE / NN_BOX;         // boxes staged at a time
+static_assert(NN_BOX == 32 && NN_TILE == NN_THREADS, "a warp stages a box");
+
+__device__ __forceinline__ float warp_min(float v)
+{
+    for (int o = 16; o > 0; o >>= 1) v = fminf(v, __shfl_xor_sync(0xffffffffu, v, o));
+    return v;
+}
+
+__device__ __forceinline__ float warp_max(float v)
+{
+    for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
+    return v;
+}
+
+// v rounded to the nearest float (a tie away from zero): on the integer pipe,
+// because an FP64 conversion takes the FP64 pipe 68 clocks
+__device__ __forceinline__ float nearest_float(double v)
+{
+    float hi, lo;
+    if (split_pair(v, hi, lo)) return hi;
+    return v == 0.0 ? 0.0f : __double2float_rn(v);
+}
+
+// floats below and above whatever rounds to f (not a number for infinite f)
+__device__ __forceinline__ float below(float f) { return f - (fabsf(f) * 1.2e-7f + 1e-44f); }
+__device__ __forceinline__ float above(float f) { return f + (fabsf(f) * 1.2e-7f + 1e-44f); }
+
+// boxes[2 k], boxes[2 k + 1]: lower and upper corner of force points
+// [32 k, 32 k + 32), rounded outward (NaN coordinates left out: such a point is
+// never a nearest neighbour)
+__global__ void __launch_bounds__(256)
+    k_nn_boxes(int64_t N, const D4 *__restrict__ x, float4 *__restrict__ boxes)
+{
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const float inf = __int_as_float(0x7f800000);
+    float4 lo = make_float4(inf, inf, inf, 0.0f), hi = make_float4(-inf, -inf, -inf, 0.0f);
+    if (i < N) {
+        const D4 p = x[i];
+        lo = make_float4(fminf(__double2float_rd(p.x), inf), fminf(__double2float_rd(p.y), inf),
+                         fminf(__double2float_rd(p.z), inf), 0.0f);
+        hi = make_float4(fmaxf(__double2float_ru(p.x), -inf), fmaxf(__double2float_ru(p.y), -inf),
+                         fmaxf(__double2float_ru(p.z), -inf), 0.0f);
+    }
+    lo = make_float4(warp_min(lo.x), warp_min(lo.y), warp_min(lo.z), 0.0f);
+    hi = make_float4(warp_max(hi.x), warp_max(hi.y), warp_max(hi.z), 0.0f);
+    if ((threadIdx.x & 31) == 0 && i < N) {
+        boxes[2 * (i / NN_BOX)] = lo;
+        boxes[2 * (i / NN_BOX) + 1] = hi;
+    }
+}
 
 // The NN_SPLIT threads of a quadrature point are consecutive lanes; each scans
 // the candidates i = sub, sub + NN_SPLIT, ... of every tile in ascending order,
@@ -119,87 +188,298 @@ constexpr int NN_TILE = 512;
 __global__ void __launch_bounds__(NN_THREADS)
     k_nearest(const NNTask *__restrict__ tasks, const int64_t *__restrict__ n_off, int nbodies,
               int global, const D4 *__restrict__ x, const D4 *__restrict__ X,
-              int32_t *__restrict__ nn, int32_t *status)
+              const float4 *__restrict__ boxes, int32_t *__restrict__ nn, int32_t *status)
 {
+    constexpr int WARPS = NN_THREADS / 32, WORDS = NN_THREADS / 32;
     __shared__ float4 tile[NN_TILE];
+    __shared__ int32_t list[NN_THREADS];         // boxes of a chunk that some warp kept, ascending
+    __shared__ unsigned int mask[WARPS][WORDS];  // each warp's kept boxes of the chunk
     __shared__ unsigned int s_cmax;
+    __shared__ int s_cnt[WARPS];
     const NNTask t = tasks[blockIdx.x];
     const int64_t n_lo = global ? 0 : n_off[t.body];
     const int64_t n_hi = global ? n_off[nbodies] : n_off[t.body + 1];
-    const int sub = threadIdx.x % NN_SPLIT;
-    const int64_t q = (int64_t)t.q0 + threadIdx.x / NN_SPLIT;
+    const int64_t b_lo = n_lo / NN_BOX, b_hi = ceil_div(n_hi, NN_BOX);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int sub = tid % NN_SPLIT;
+    const int64_t q = (int64_t)t.q0 + tid / NN_SPLIT;
     const bool active = q < t.q1;
+    const float inf = __int_as_float(0x7f800000), nan = __int_as_float(0x7fffffff);
     double qx = 0.0, qy = 0.0, qz = 0.0;
+    float4 ql = make_float4(inf, inf, inf, 0.0f), qh = make_float4(-inf, -inf, -inf, 0.0f);
     if (active) {
         D4 p = X[q];
         qx = p.x;
         qy = p.y;
         qz = p.z;
     }
-    const float fx = __double2float_rn(qx), fy = __double2float_rn(qy), fz = __double2float_rn(qz);
-    if (threadIdx.x == 0) s_cmax = 0u;
-    float best = __int_as_float(0x7f800000);
-
-    for (int64_t base = n_lo; base < n_hi; base += NN_TILE) {
-        const int cnt = (int)min((int64_t)NN_TILE, n_hi - base);
-        __syncthreads();
-        float lmax = 0.0f;
-        for (int i = threadIdx.x; i < cnt; i += NN_THREADS) {
-            D4 p = x[base + i];
-            float4 v = make_float4(__double2float_rn(p.x), __double2float_rn(p.y),
-                                   __double2float_rn(p.z), 0.0f);
-            tile[i] = v;
-            lmax = fmaxf(lmax, fmaxf(fabsf(v.x), fmaxf(fabsf(v.y), fabsf(v.z))));
+    const float fx = nearest_float(qx), fy = nearest_float(qy), fz = nearest_float(qz);
+    if (active) {
+        ql = make_float4(below(fx), below(fy), below(fz), 0.0f);
+        qh = make_float4(above(fx), above(fy), above(fz), 0.0f);
+    }
+    if (tid == 0) s_cmax = 0u;
+    // the box of the warp's quadrature points
+    ql = make_float4(warp_min(ql.x), warp_min(ql.y), warp_min(ql.z), 0.0f);
+    qh = make_float4(warp_max(qh.x), warp_max(qh.y), warp_max(qh.z), 0.0f);
+    // the box whose centre is closest: lexicographic minimum of (distance, index)
+    int64_t seed;
+    {
+        unsigned key = 0xffffffffu, at = 0u;
+        for (int64_t k = b_lo + lane; k < b_hi; k += 32) {
+            const float4 l = boxes[2 * k], h = boxes[2 * k + 1];
+            const float cx = (l.x + h.x) - (ql.x + qh.x), cy = (l.y + h.y) - (ql.y + qh.y);
+            const float cz = (l.z + h.z) - (ql.z + qh.z);
+            const unsigned d = __float_as_uint(cx * cx + cy * cy + cz * cz) & 0x7fffffffu;
+            if (d < key) {
+                key = d;
+                at = (unsigned)(k - b_lo);
+            }
         }
-        for (int o = 16; o > 0; o >>= 1) lmax = fmaxf(lmax, __shfl_xor_sync(0xffffffffu, lmax, o));
-        if ((threadIdx.x & 31) == 0) atomicMax(&s_cmax, __float_as_uint(lmax));
-        __syncthreads();
+        const unsigned wk = __reduce_min_sync(0xffffffffu, key);
+        seed = b_lo + __reduce_min_sync(0xffffffffu, key == wk ? at : 0xffffffffu);
+    }
+    float best = inf;
+    __syncthreads();  // s_cmax is set
+    // box k into this warp's slice of the tile
+    auto stage = [&](int64_t k) {
+        const int64_t i = k * NN_BOX + lane;
+        float4 v = make_float4(nan, nan, nan, 0.0f);
+        float lmax = 0.0f;
+        if (i >= n_lo && i < n_hi) {
+            const D4 p = x[i];
+            v = make_float4(nearest_float(p.x), nearest_float(p.y), nearest_float(p.z), 0.0f);
+            lmax = fmaxf(fabsf(v.x), fmaxf(fabsf(v.y), fabsf(v.z)));
+        }
+        tile[tid] = v;
+        lmax = warp_max(lmax);
+        if (lane == 0) atomicMax(&s_cmax, __float_as_uint(lmax));
+    };
+    auto scan = [&](int slot) {
         if (active) {
-#pragma unroll 8
-            for (int i = sub; i < cnt; i += NN_SPLIT) {
-                float4 v = tile[i];
-                float dx = v.x - fx, dy = v.y - fy, dz = v.z - fz;
-                float d2 = dx * dx + dy * dy + dz * dz;
-                best = fminf(best, d2);
+#pragma unroll
+            for (int i = sub; i < NN_BOX; i += NN_SPLIT) {
+                const float4 v = tile[slot * NN_BOX + i];
+                const float dx = v.x - fx, dy = v.y - fy, dz = v.z - fz;
+                best = fminf(best, dx * dx + dy * dy + dz * dz);
+            }
+        }
+    };
+    // the squared bound above for the smallest distance so far, and 1e-43 for the
+    // absolute rounding of squares that are subnormal (distances below 1e-19)
+    auto bound = [&]() {
+#pragma unroll
+        for (int o = 1; o < NN_SPLIT; o <<= 1)
+            best = fminf(best, __shfl_xor_sync(0xffffffffu, best, o));
+        const float cmax =
+            fmaxf(__uint_as_float(s_cmax), fmaxf(fabsf(fx), fmaxf(fabsf(fy), fabsf(fz))));
+        const float e = 4.2e-7f * cmax;
+        const float th = (sqrtf(best) * (1.0f + 1e-6f) + 2.0f * e + 1e-30f) * (1.0f + 1e-6f);
+        return th * th + 1e-43f;
+    };
+    // the largest of the warp's bounds (a point that is not a number has none)
+    auto warp_bound = [&](float th) {
+        return __uint_as_float(
+            __reduce_max_sync(0xffffffffu, active && th >= 0.0f ? __float_as_uint(th) : 0u));
+    };
+    // each quadrature point's own closest box (by centre), evaluated for it: for
+    // warps whose points lie far apart, which one box serves badly
+    auto seed_each = [&]() {
+        unsigned key = 0xffffffffu, at = 0u;
+        for (int64_t k = b_lo + sub; k < b_hi; k += NN_SPLIT) {
+            const float4 l = boxes[2 * k], h = boxes[2 * k + 1];
+            const float cx = (l.x + h.x) - 2.0f * fx, cy = (l.y + h.y) - 2.0f * fy;
+            const float cz = (l.z + h.z) - 2.0f * fz;
+            const unsigned d = __float_as_uint(cx * cx + cy * cy + cz * cz) & 0x7fffffffu;
+            if (d < key) {
+                key = d;
+                at = (unsigned)(k - b_lo);
+            }
+        }
+#pragma unroll
+        for (int o = 1; o < NN_SPLIT; o <<= 1) {
+            const unsigned ok = __shfl_xor_sync(0xffffffffu, key, o);
+            const unsigned oa = __shfl_xor_sync(0xffffffffu, at, o);
+            if (ok < key || (ok == key && oa < at)) {
+                key = ok;
+                at = oa;
+            }
+        }
+        for (int j = 0; j < 32 / NN_SPLIT; ++j) {
+            stage(b_lo + __shfl_sync(0xffffffffu, at, NN_SPLIT * j));
+            __syncwarp();
+            if (lane / NN_SPLIT == j) scan(warp);
+            __syncwarp();
+        }
+    };
+    constexpr int NN_MANY = 16;  // kept boxes of a chunk from which on each point is asked
+    bool seeded = false;
+    // keeps, of the chunk of NN_THREADS boxes from k0 on, those within th of one
+    // of the warp's points; returns how many some warp of the block kept
+    auto keep = [&](int64_t k0, float &th) {
+        const int words = (int)min((int64_t)WORDS, ceil_div(b_hi - k0, 32));
+        const float u2 = warp_bound(th);
+        unsigned mine = 0u;
+        for (int w = 0; w < words; ++w) {
+            const int64_t k = k0 + 32 * w + lane;
+            bool in = false;
+            if (k < b_hi) {
+                const float4 l = boxes[2 * k], h = boxes[2 * k + 1];
+                const float dx = fmaxf(0.0f, fmaxf(l.x - qh.x, ql.x - h.x));
+                const float dy = fmaxf(0.0f, fmaxf(l.y - qh.y, ql.y - h.y));
+                const float dz = fmaxf(0.0f, fmaxf(l.z - qh.z, ql.z - h.z));
+                in = !((dx * dx + dy * dy + dz * dz) * (1.0f - 1e-6f) > u2);
+            }
+            const unsigned bal = __ballot_sync(0xffffffffu, in);
+            if (lane == w) mine = bal;
+        }
+        if (__reduce_add_sync(0xffffffffu, __popc(mine)) > NN_MANY) {
+            // (in the first chunk, where no other warp looks at this one's slice of
+            // the tile)
+            if (!seeded && k0 == b_lo) {
+                seed_each();
+                th = bound();
+                seeded = true;
+            }
+            for (int w = 0; w < words; ++w) {
+                const int64_t k = k0 + 32 * w + lane;
+                bool in = (__shfl_sync(0xffffffffu, mine, w) >> lane) & 1u;
+                if (!__any_sync(0xffffffffu, in)) continue;
+                float4 l = make_float4(0.0f, 0.0f, 0.0f, 0.0f), h = l;
+                if (in) {
+                    l = boxes[2 * k];
+                    h = boxes[2 * k + 1];
+                }
+                bool any = false;
+                for (int j = 0; j < 32 / NN_SPLIT; ++j) {
+                    const float px = __shfl_sync(0xffffffffu, fx, NN_SPLIT * j);
+                    const float py = __shfl_sync(0xffffffffu, fy, NN_SPLIT * j);
+                    const float pz = __shfl_sync(0xffffffffu, fz, NN_SPLIT * j);
+                    const float pt = __shfl_sync(0xffffffffu, active ? th : -1.0f, NN_SPLIT * j);
+                    const float dx = fmaxf(0.0f, fmaxf(l.x - above(px), below(px) - h.x));
+                    const float dy = fmaxf(0.0f, fmaxf(l.y - above(py), below(py) - h.y));
+                    const float dz = fmaxf(0.0f, fmaxf(l.z - above(pz), below(pz) - h.z));
+                    any |= !((dx * dx + dy * dy + dz * dz) * (1.0f - 1e-6f) > pt) && !(pt < 0.0f);
+                }
+                const unsigned bal = __ballot_sync(0xffffffffu, in && any);
+                if (lane == w) mine = bal;
+            }
+        }
+        __syncthreads();  // everyone is done with the list, the masks and the tile
+        if (lane < WORDS) mask[warp][lane] = mine;
+        __syncthreads();
+        unsigned any = 0u;  // word `warp` of the union
+        for (int w = 0; w < WARPS; ++w) any |= mask[w][warp];
+        if (lane == 0) s_cnt[warp] = __popc(any);
+        __syncthreads();
+        int before = 0, total = 0;
+        for (int w = 0; w < WARPS; ++w) {
+            if (w < warp) before += s_cnt[w];
+            total += s_cnt[w];
+        }
+        if ((any >> lane) & 1u) list[before + __popc(any & ((1u << lane) - 1u))] = tid;
+        __syncthreads();
+        return total;
+    };
+    auto kept_by_me = [&](int r) { return (mask[warp][r >> 5] >> (r & 31)) & 1u; };
+
+    if (b_hi > b_lo) {
+        stage(seed);
+        __syncwarp();
+        scan(warp);
+    }
+    float th = bound();
+    const bool one_chunk = b_hi - b_lo <= NN_THREADS;
+    int kept = 0;
+    for (int64_t k0 = b_lo; k0 < b_hi; k0 += NN_THREADS) {
+        kept = keep(k0, th);
+        for (int j = 0; j < kept; j += NN_BOXES) {
+            if (j) __syncthreads();  // the previous boxes are scanned
+            const int cnt = min(NN_BOXES, kept - j);
+            if (warp < cnt) stage(k0 + list[j + warp]);
+            __syncthreads();
+            for (int s = 0; s < cnt; ++s)
+                if (kept_by_me(list[j + s])) scan(s);
+        }
+        if (!one_chunk) th = bound();
+    }
+    __syncthreads();  // s_cmax is final
+    th = bound();
+
+    // this lane's candidates: how many, and the first four (from n_lo on)
+    int found = 0;
+    int32_t cand[4] = {0, 0, 0, 0};
+    auto decide = [&](int slot, int64_t k) {
+        if (active) {
+#pragma unroll
+            for (int i = sub; i < NN_BOX; i += NN_SPLIT) {
+                const float4 v = tile[slot * NN_BOX + i];
+                const float dx = v.x - fx, dy = v.y - fy, dz = v.z - fz;
+                const float d2 = dx * dx + dy * dy + dz * dz;
+                if (d2 <= th) {
+                    const int32_t n = (int32_t)(k * NN_BOX + i - n_lo);
+                    if (found == 0) cand[0] = n;
+                    if (found == 1) cand[1] = n;
+                    if (found == 2) cand[2] = n;
+                    if (found == 3) cand[3] = n;
+                    ++found;
+                }
+            }
+        }
+    };
+    if (one_chunk && kept <= NN_BOXES) {
+        // the tile still holds them all
+        for (int s = 0; s < kept; ++s)
+            if (kept_by_me(list[s])) decide(s, b_lo + list[s]);
+    } else {
+        seeded = true;  // every distance is known: th stays
+        for (int64_t k0 = b_lo; k0 < b_hi; k0 += NN_THREADS) {
+            kept = keep(k0, th);
+            for (int j = 0; j < kept; j += NN_BOXES) {
+                if (j) __syncthreads();
+                const int cnt = min(NN_BOXES, kept - j);
+                if (warp < cnt) stage(k0 + list[j + warp]);
+                __syncthreads();
+                for (int s = 0; s < cnt; ++s)
+                    if (kept_by_me(list[j + s])) decide(s, k0 + list[j + s]);
             }
         }
     }
+    // One candidate in all, at a finite distance, is the neighbour; more are
+    // decided in FP64 (76 clocks of the pipe an operation: only then).
+    int total = found, most = found;
 #pragma unroll
-    for (int o = 1; o < NN_SPLIT; o <<= 1) best = fminf(best, __shfl_xor_sync(0xffffffffu, best, o));
-    __syncthreads();
-    const float cmax =
-        fmaxf(__uint_as_float(s_cmax), fmaxf(fabsf(fx), fmaxf(fabsf(fy), fabsf(fz))));
-    const float e = 4.2e-7f * cmax;
-    float th = (sqrtf(best) * (1.0f + 1e-6f) + 2.0f * e + 1e-30f) * (1.0f + 1e-6f);
-    th = th * th;
-
+    for (int o = 1; o < NN_SPLIT; o <<= 1) {
+        total += __shfl_xor_sync(0xffffffffu, total, o);
+        most = max(most, __shfl_xor_sync(0xffffffffu, most, o));
+    }
     double best64 = __longlong_as_double(0x7ff0000000000000LL);
     int64_t arg = -1;
-    for (int64_t base = n_lo; base < n_hi; base += NN_TILE) {
-        const int cnt = (int)min((int64_t)NN_TILE, n_hi - base);
-        __syncthreads();
-        for (int i = threadIdx.x; i < cnt; i += NN_THREADS) {
-            D4 p = x[base + i];
-            tile[i] = make_float4(__double2float_rn(p.x), __double2float_rn(p.y),
-                                  __double2float_rn(p.z), 0.0f);
+    auto try64 = [&](int64_t n) {
+        const D4 p = x[n];
+        double ex = __dsub_rn(p.x, qx), ey = __dsub_rn(p.y, qy), ez = __dsub_rn(p.z, qz);
+        double s = __dadd_rn(__dadd_rn(__dmul_rn(ex, ex), __dmul_rn(ey, ey)), __dmul_rn(ez, ez));
+        if (s < best64) {
+            best64 = s;
+            arg = n;
         }
-        __syncthreads();
-        if (active) {
-            for (int i = sub; i < cnt; i += NN_SPLIT) {
-                float4 v = tile[i];
-                float dx = v.x - fx, dy = v.y - fy, dz = v.z - fz;
-                float d2 = dx * dx + dy * dy + dz * dz;
-                if (d2 <= th) {
-                    D4 p = x[base + i];
-                    double ex = __dsub_rn(p.x, qx), ey = __dsub_rn(p.y, qy), ez = __dsub_rn(p.z, qz);
-                    double s = __dadd_rn(__dadd_rn(__dmul_rn(ex, ex), __dmul_rn(ey, ey)),
-                                         __dmul_rn(ez, ez));
-                    if (s < best64) {
-                        best64 = s;
-                        arg = base + i;
-                    }
-                }
-            }
+    };
+    if (total == 1 && best < inf) {
+        if (found) {
+            arg = n_lo + cand[0];
+            best64 = 0.0;
+        }
+    } else if (most <= 4) {
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+            if (c < found) try64(n_lo + cand[c]);
+    } else {
+        // many at nearly the same distance: every force point again
+        for (int64_t n = n_lo + sub; n < n_hi; n += NN_SPLIT) {
+            const D4 p = x[n];
+            const float dx = nearest_float(p.x) - fx, dy = nearest_float(p.y) - fy;
+            const float dz = nearest_float(p.z) - fz;
+            if (dx * dx + dy * dy + dz * dz <= th) try64(n);
         }
     }
 #pragma unroll
@@ -223,10 +503,11 @@ void launch_nearest(Ctx &c, const D4 *x, const D4 *Xw, int32_t *nn, bool only_de
     int count = only_deforming ? c.n_tasks_deform : c.n_tasks_all;
     if (count == 0) return;
     c.tbeg(PH_NEAREST);
+    k_nn_boxes<<<(unsigned)ceil_div(c.N, 256), 256, 0, c.stream>>>(c.N, x, c.d_nn_box);
     k_nearest<<<count, NN_THREADS, 0, c.stream>>>(tasks, c.d_n_off, c.nbodies, c.nn_global, x, Xw,
-                                                   nn, c.d_status);
+                                                   c.d_nn_box, nn, c.d_status);
     c.tend(PH_NEAREST);
-    c.launches += 1;
+    c.launches += 2;
 }
 
 // ---------------------------------------------------------------------------
@@ -245,34 +526,56 @@ __global__ void k_count(int64_t Q, int64_t N, const int32_t *__restrict__ nn,
     }
 }
 
-// Exclusive scan of cnt[0..N) into seg_ptr[0..N] (single block of 1024).
+// Exclusive scan of cnt[0..N) into seg_ptr[0..N] and cursor[0..N] (one block of
+// 1024 threads; cnt may alias cursor).  A warp takes 256 consecutive counts as
+// 8 rows of 32, so that every access is coalesced.
 __global__ void __launch_bounds__(1024)
     k_scan(int64_t N, const int32_t *cnt, int32_t *__restrict__ seg_ptr, int32_t *cursor)
 {
-    __shared__ int32_t part[1024];
-    const int tid = threadIdx.x;
-    const int64_t chunk = ceil_div(N, 1024);
-    const int64_t lo = min(N, tid * chunk), hi = min(N, lo + chunk);
-    int32_t s = 0;
-    for (int64_t i = lo; i < hi; ++i) s += cnt[i];
-    part[tid] = s;
-    __syncthreads();
-    for (int off = 1; off < 1024; off <<= 1) {
-        int32_t v = tid >= off ? part[tid - off] : 0;
+    __shared__ int32_t part[32];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    int32_t run = 0;  // sum of the tiles before
+    for (int64_t base = 0; base < N; base += 8192) {
+        const int64_t i0 = base + 256 * warp + lane;
+        int32_t v[8], inc[8];
+#pragma unroll
+        for (int r = 0; r < 8; ++r) inc[r] = v[r] = i0 + 32 * r < N ? cnt[i0 + 32 * r] : 0;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1)
+#pragma unroll
+            for (int r = 0; r < 8; ++r) {
+                const int32_t u = __shfl_up_sync(0xffffffffu, inc[r], o);
+                if (lane >= o) inc[r] += u;
+            }
+        int32_t sum = 0;  // of the warp's rows before
+#pragma unroll
+        for (int r = 0; r < 8; ++r) {
+            const int32_t t = __shfl_sync(0xffffffffu, inc[r], 31);
+            inc[r] += sum - v[r];
+            sum += t;
+        }
+        if (lane == 31) part[warp] = sum;
         __syncthreads();
-        part[tid] += v;
-        __syncthreads();
+        int32_t w = part[lane];
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int32_t u = __shfl_up_sync(0xffffffffu, w, o);
+            if (lane >= o) w += u;
+        }
+        const int32_t before = __shfl_sync(0xffffffffu, w, max(warp - 1, 0));
+        const int32_t at = run + (warp ? before : 0);
+#pragma unroll
+        for (int r = 0; r < 8; ++r)
+            if (i0 + 32 * r < N) {
+                seg_ptr[i0 + 32 * r] = at + inc[r];
+                cursor[i0 + 32 * r] = at + inc[r];
+            }
+        run += __shfl_sync(0xffffffffu, w, 31);
+        __syncthreads();  // part is free for the next tile
     }
-    int32_t run = tid ? part[tid - 1] : 0;
-    for (int64_t i = lo; i < hi; ++i) {
-        int32_t ci = cnt[i];  // cnt may alias cursor: read before overwriting
-        seg_ptr[i] = run;
-        cursor[i] = run;
-        run += ci;
-    }
-    if (tid == 1023) {
-        seg_ptr[N] = part[1023];
-        cursor[N] = part[1023];
+    if (tid == 0) {
+        seg_ptr[N] = run;
+        cursor[N] = run;
     }
 }
 
@@ -288,13 +591,25 @@ __global__ void k_scatter(int64_t Q, int64_t N, const int32_t *__restrict__ nn,
     }
 }
 
-// Order each segment by ascending q (insertion sort; segments hold ~Q/N points).
+// Order each segment by ascending q.  Segments hold about Q / N points: a warp
+// ranks up to 32 (each lane counts the smaller values by shuffles; one thread
+// per segment with an insertion sort in global memory took 24 us for 9200
+// segments), its first lane sorts a longer one by insertion.
 __global__ void k_sort_segments(int64_t N, const int32_t *__restrict__ seg_ptr,
                                 int32_t *__restrict__ perm)
 {
-    int64_t n = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int64_t n = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / 32;
     if (n >= N) return;
-    int32_t lo = seg_ptr[n], hi = seg_ptr[n + 1];
+    const int lane = threadIdx.x & 31;
+    const int32_t lo = seg_ptr[n], hi = seg_ptr[n + 1], len = hi - lo;
+    if (len <= 32) {
+        const int32_t v = lane < len ? perm[lo + lane] : 0;
+        int rank = 0;
+        for (int k = 0; k < len; ++k) rank += __shfl_sync(0xffffffffu, v, k) < v;
+        if (lane < len) perm[lo + rank] = v;
+        return;
+    }
+    if (lane) return;
     for (int32_t i = lo + 1; i < hi; ++i) {
         int32_t v = perm[i];
         int32_t j = i - 1;
@@ -317,7 +632,8 @@ void launch_segments(Ctx &c, const int32_t *nn, int32_t *seg_ptr, int32_t *perm)
     k_scan<<<1, 1024, 0, c.stream>>>(c.N, c.d_cursor, seg_ptr, c.d_cursor);
     k_scatter<<<(unsigned)ceil_div(c.Q, threads), threads, 0, c.stream>>>(c.Q, c.N, nn, c.d_cursor,
                                                                           perm);
-    k_sort_segments<<<(unsigned)ceil_div(c.N, threads), threads, 0, c.stream>>>(c.N, seg_ptr, perm);
+    k_sort_segments<<<(unsigned)ceil_div(32 * c.N, threads), threads, 0, c.stream>>>(c.N, seg_ptr,
+                                                                                      perm);
     c.tend(PH_SEGMENTS);
     c.launches += 4;
 }

@@ -46,6 +46,7 @@ struct NNTask {
 constexpr int NN_QPB = 128;
 constexpr int NN_SPLIT = 4;
 constexpr int NN_THREADS = NN_QPB * NN_SPLIT;
+constexpr int NN_BOX = 32;  // force points of a bounding box
 
 struct Ctx;
 
@@ -194,6 +195,7 @@ struct Ctx {
     double *d_x0 = nullptr, *d_B = nullptr, *d_x0_save = nullptr, *d_B_save = nullptr;
     NNTask *d_tasks_all = nullptr, *d_tasks_deform = nullptr;
     int n_tasks_all = 0, n_tasks_deform = 0;
+    float4 *d_nn_box = nullptr;  // boxes of 32 force points each (lower, upper corner)
     bool nn_valid = false;
 
     // clouds and right-hand side (lab frame)

@@ -7,7 +7,7 @@
 // synchronise the device, or a process that reserved all device memory up
 // front.  This entry point takes the caller's inputs and outputs and keeps its
 // scratch (segment counters and cursors, the block task table, the body
-// offsets and a status word) in file-scope __device__ arrays of a fixed size,
+// offsets, the force points' boxes and a status word) in file-scope __device__ arrays of a fixed size,
 // which every GPU that loads the library holds until the process exits.
 //
 // The kernels are the ones nrs_nearest_build runs (geometry.cu); nothing in
@@ -19,8 +19,10 @@
 namespace nrs {
 
 // kernels defined in geometry.cu
+__global__ void k_nn_boxes(int64_t N, const D4 *x, float4 *boxes);
 __global__ void k_nearest(const NNTask *tasks, const int64_t *n_off, int nbodies, int global,
-                          const D4 *x, const D4 *X, int32_t *nn, int32_t *status);
+                          const D4 *x, const D4 *X, const float4 *boxes, int32_t *nn,
+                          int32_t *status);
 __global__ void k_count(int64_t Q, int64_t N, const int32_t *nn, int32_t *cnt);
 __global__ void k_scan(int64_t N, const int32_t *cnt, int32_t *seg_ptr, int32_t *cursor);
 __global__ void k_scatter(int64_t Q, int64_t N, const int32_t *nn, int32_t *cursor, int32_t *perm);
@@ -41,6 +43,7 @@ static __device__ __align__(256) NNTask g_tasks[kMaxTasks];
 static __device__ __align__(256) int64_t g_n_off[kMaxBodies + 1];
 static __device__ __align__(256) int64_t g_q_off[kMaxBodies + 1];
 static __device__ __align__(256) int32_t g_status[1];
+static __device__ __align__(256) float4 g_box[2 * (kMaxN / NN_BOX)];
 
 struct DevScratch {
     bool ready = false;
@@ -49,6 +52,7 @@ struct DevScratch {
     int64_t *n_off = nullptr;
     int64_t *q_off = nullptr;
     int32_t *status = nullptr;
+    float4 *box = nullptr;
 };
 
 constexpr int kMaxDevices = 64;
@@ -68,6 +72,7 @@ cudaError_t setup_device(int dev, DevScratch **out)
         if ((e = cudaGetSymbolAddress((void **)&s.n_off, g_n_off)) != cudaSuccess) return e;
         if ((e = cudaGetSymbolAddress((void **)&s.q_off, g_q_off)) != cudaSuccess) return e;
         if ((e = cudaGetSymbolAddress((void **)&s.status, g_status)) != cudaSuccess) return e;
+        if ((e = cudaGetSymbolAddress((void **)&s.box, g_box)) != cudaSuccess) return e;
         s.ready = true;
     }
     *out = &s;
@@ -121,13 +126,15 @@ extern "C" nrs_status nrs_nearest_build_static(const double *x, const double *Xw
         cudaMemsetAsync(perm, 0, sizeof(int32_t) * Q, st) != cudaSuccess)
         return NRS_ECUDA;
     k_static_tasks<<<1, 1, 0, st>>>(nbodies, s->q_off, s->tasks);
-    k_nearest<<<(unsigned)ntasks, NN_THREADS, 0, st>>>(s->tasks, s->n_off, nbodies, global ? 1 : 0,
-                                                 (const D4 *)x, (const D4 *)Xw, nn, s->status);
     const int threads = 256;
+    k_nn_boxes<<<(unsigned)ceil_div(N, threads), threads, 0, st>>>(N, (const D4 *)x, s->box);
+    k_nearest<<<(unsigned)ntasks, NN_THREADS, 0, st>>>(s->tasks, s->n_off, nbodies, global ? 1 : 0,
+                                                 (const D4 *)x, (const D4 *)Xw, s->box, nn,
+                                                 s->status);
     k_count<<<(unsigned)ceil_div(Q, threads), threads, 0, st>>>(Q, N, nn, s->cursor);
     k_scan<<<1, 1024, 0, st>>>(N, s->cursor, seg_ptr, s->cursor);
     k_scatter<<<(unsigned)ceil_div(Q, threads), threads, 0, st>>>(Q, N, nn, s->cursor, perm);
-    k_sort_segments<<<(unsigned)ceil_div(N, threads), threads, 0, st>>>(N, seg_ptr, perm);
+    k_sort_segments<<<(unsigned)ceil_div(32 * N, threads), threads, 0, st>>>(N, seg_ptr, perm);
     if (cudaGetLastError() != cudaSuccess) return NRS_ECUDA;
     // the device status word (ST_NONFINITE: a non-finite coordinate; those
     // quadrature points have nn < 0 and belong to no segment) to the caller's

@@ -138,16 +138,23 @@ NRS_HD Sig mul_sig(const Sig &a, uint64_t b2, uint32_t bf, bool &tie)
     return r;
 }
 
-// s = RN(1 / RN(rho RN(sqrt(rho)))) for rho in [2^-100, 2^100]; `tie` as above.
-NRS_HD Sig inv_rho_sqrt(double rho_d, bool &tie)
+// 1/sqrt of rho in [2^-100, 2^100) to 2^-28: rho = m' 2^(2k) with m' in [1, 4).
+struct RsqrtSeed {
+    uint64_t M;    // m' 2^62
+    uint32_t Y;    // 2^30 / sqrt(m'), about
+    uint32_t ex;   // rho's biased exponent, 1024 + 2k - par
+    uint32_t par;  // 1: m' below 2
+};
+
+NRS_HD RsqrtSeed rsqrt_seed(double rho_d)
 {
     const uint64_t rb = double_bits(rho_d);
     const uint32_t rhi = hi32(rb), rlo = lo32(rb);
-    const Sig rho = unpack(rho_d);
-    // rho = m' 2^(2k), m' in [1, 4); par = 1: m' below 2
-    const uint32_t ex = rhi >> 20, par = ex & 1u;
-    const uint64_t M = rho.m << (11 - par);  // m' 2^62
-    const uint32_t Mh = hi32(M);
+    RsqrtSeed r;
+    r.ex = rhi >> 20;
+    r.par = r.ex & 1u;
+    r.M = unpack(rho_d).m << (11 - r.par);
+    const uint32_t Mh = hi32(r.M);
     // y0 = 1/sqrt(m') to 16 bits, truncated: the seed's operand is rounded to
     // mid-interval at 2^-20 so that y stays inside (1/2, 1)
     const uint32_t fb = (funnel_l(rlo, rhi - (896u << 20), 3) & ~0x1fu) | 0x10u;
@@ -157,7 +164,34 @@ NRS_HD Sig inv_rho_sqrt(double rho_d, bool &tie)
     const int32_t e = (int32_t)(0u - (uint32_t)(W >> 18));
     const uint32_t e2 = hi32((uint64_t)((int64_t)e * e));  // e0^2 2^56
     const int32_t c = e + (int32_t)((e2 * 3u) >> 14);      // in units of 2^-45
-    const uint32_t Y = (Y0 << 14) + (uint32_t)(((int64_t)(int32_t)Y0 * c) >> 31);  // y 2^30
+    r.Y = (Y0 << 14) + (uint32_t)(((int64_t)(int32_t)Y0 * c) >> 31);
+    return r;
+}
+
+// y^2 and y^3, rounded, for one y within 2^-28 of 1/sqrt(rho), rho in
+// [2^-100, 2^100): with e = 1 - rho y^2, rho^(-3/2) = y^3 (1 + 3/2 e) to 2^-54.
+NRS_HD void rsqrt_powers(double rho, double &y2, double &y3)
+{
+    const RsqrtSeed r = rsqrt_seed(rho);
+    const uint32_t Y = r.Y < 0x3fffffffu ? r.Y : 0x3fffffffu;  // below 2^30
+    const uint64_t v = wide(Y, Y, 0);                          // y^2 2^60, 59 or 60 bits
+    const uint32_t top = hi32(v) >> 27;
+    const uint32_t k2 = r.ex + r.par;                          // 1024 + 2k
+    y2 = bits_double(((v + (32ull << top)) >> (6u + top)) + ((uint64_t)(1021u + 1024u - 1u + top - k2) << 52));
+    const uint64_t h = wide(hi32(v), Y, hi32(wide(lo32(v), Y, 0)));  // y^3 2^58, 56 to 58 bits
+    const uint32_t n = (hi32(h) >> 25) ? 2u : (hi32(h) >> 24) ? 1u : 0u;  // bits above 56
+    // 2^52 of the significand is bit 55 + n of h: value m 2^(3 + n - 58 - 3k)
+    y3 = bits_double(((h + (4ull << n)) >> (3u + n)) +
+                     ((uint64_t)(1023u + 52u + 3u + n - 58u - 1u - (3 * (k2 - 1024u)) / 2) << 52));
+}
+
+// s = RN(1 / RN(rho RN(sqrt(rho)))) for rho in [2^-100, 2^100); `tie` as above.
+NRS_HD Sig inv_rho_sqrt(double rho_d, bool &tie)
+{
+    const RsqrtSeed seed = rsqrt_seed(rho_d);
+    const Sig rho = unpack(rho_d);
+    const uint64_t M = seed.M;
+    const uint32_t Mh = hi32(M), Y = seed.Y, ex = seed.ex, par = seed.par;
     // g = sqrt(m') to about 2^-28, then one step g + (m' - g^2) y / 2
     const uint32_t G = (uint32_t)(wide(Mh, Y, 0) >> 29);  // g 2^31
     const int64_t d = (int64_t)(M - wide(G, G, 0));       // (m' - g^2) 2^62

@@ -33,7 +33,6 @@ enum {
     SC_OUTER_DONE = 4,
     SC_RN = 5,
     SC_BN = 6,
-    SC_AN = 7,
     SC_RES = 8,
     SC_DNPREV = 10,
     SC_STAG = 11,  // the last correction did not halve
@@ -191,11 +190,17 @@ __global__ void __launch_bounds__(NB)
 
 constexpr int MV_THREADS = 128;
 
-// part[s*n + i] = sum_{j in split s} A[i,j] v[j] (|A[i,j]| when ABS) for the
-// FP64 matrix.  Each thread owns two adjacent rows (one 16-byte load per
-// column), so a warp reads 512 contiguous bytes per column; rows i+1 >= n read
-// the padding rows below n (allocated, results discarded).
-template <bool ABS>
+// max of non-negative values into *p (their bits order as integers)
+__device__ __forceinline__ void atomic_max_nonneg(double *p, double v)
+{
+    atomicMax(reinterpret_cast<unsigned long long *>(p),
+              (unsigned long long)__double_as_longlong(v));
+}
+
+// part[s*n + i] = sum_{j in split s} A[i,j] v[j] for the FP64 matrix.  Each
+// thread owns two adjacent rows (one 16-byte load per column), so a warp reads
+// 512 contiguous bytes per column; rows i+1 >= n read the padding rows below n
+// (allocated, results discarded).
 __global__ void __launch_bounds__(MV_THREADS)
     k_gemv_part(int64_t n, const double *__restrict__ A, int64_t lda, const double *__restrict__ v,
                 double *__restrict__ part, int64_t cols_per_split)
@@ -209,14 +214,64 @@ __global__ void __launch_bounds__(MV_THREADS)
 #pragma unroll 8
     for (int64_t j = j0; j < j1; ++j) {
         const double2 x = __ldg(reinterpret_cast<const double2 *>(a + j * lda));
-        if (ABS) {
-            s0 += fabs(x.x);
-            s1 += fabs(x.y);
-        } else {
-            const double vj = __ldg(&v[j]);
-            s0 += x.x * vj;
-            s1 += x.y * vj;
+        const double vj = __ldg(&v[j]);
+        s0 += x.x * vj;
+        s1 += x.y * vj;
+    }
+    part[blockIdx.y * n + i] = s0;
+    if (i + 1 < n) part[blockIdx.y * n + i + 1] = s1;
+}
+
+// part[s*n + i] = sum_{j in split s} |A[i,j]|, laid out as k_gemv_part; `one` is
+// 1.0 (a fused multiply-add issues faster than an addition).  One more row of
+// blocks (blockIdx.y == splits) forms scal[SC_FXX] = ||x||_inf and scal[SC_BN]
+// = ||b||_inf and clears the maxima that the later kernels take by atomics.
+__global__ void __launch_bounds__(MV_THREADS)
+    k_rowsums_part(int64_t n, const double *__restrict__ A, int64_t lda, double one,
+                   const double *__restrict__ x, const double *__restrict__ b,
+                   double *__restrict__ part, int64_t cols_per_split, double *__restrict__ scal)
+{
+    if (blockIdx.y + 1 == gridDim.y) {
+        if (blockIdx.x) return;
+        __shared__ double sx[MV_THREADS / 32], sb[MV_THREADS / 32];
+        double xm = 0.0, bm = 0.0;
+#pragma unroll 4
+        for (int64_t e = threadIdx.x; e < n; e += MV_THREADS) {
+            xm = fmax(xm, fabs(x[e]));
+            bm = fmax(bm, fabs(b[e]));
         }
+        for (int o = 16; o > 0; o >>= 1) {
+            xm = fmax(xm, __shfl_xor_sync(0xffffffffu, xm, o));
+            bm = fmax(bm, __shfl_xor_sync(0xffffffffu, bm, o));
+        }
+        if ((threadIdx.x & 31) == 0) {
+            sx[threadIdx.x >> 5] = xm;
+            sb[threadIdx.x >> 5] = bm;
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            for (int w = 1; w < MV_THREADS / 32; ++w) {
+                xm = fmax(xm, sx[w]);
+                bm = fmax(bm, sb[w]);
+            }
+            scal[SC_FXX] = xm;
+            scal[SC_BN] = bm;
+            scal[SC_FXA] = 0.0;
+            scal[SC_RN] = 0.0;
+        }
+        return;
+    }
+    const int64_t i = ((int64_t)blockIdx.x * MV_THREADS + threadIdx.x) * 2;
+    const int64_t j0 = (int64_t)blockIdx.y * cols_per_split;
+    const int64_t j1 = min(n, j0 + cols_per_split);
+    if (i >= n) return;
+    double s0 = 0.0, s1 = 0.0;
+    const double *a = A + i;
+#pragma unroll 8
+    for (int64_t j = j0; j < j1; ++j) {
+        const double2 v = __ldg(reinterpret_cast<const double2 *>(a + j * lda));
+        s0 = fma(fabs(v.x), one, s0);
+        s1 = fma(fabs(v.y), one, s1);
     }
     part[blockIdx.y * n + i] = s0;
     if (i + 1 < n) part[blockIdx.y * n + i + 1] = s1;
@@ -264,11 +319,12 @@ __global__ void __launch_bounds__(MV_THREADS)
 // sum_{j in split s} fl(A[i,j] v[j]) as a 192-bit integer with the anchor of
 // ||A||_inf = scal[SC_FXA], ||v||_inf = scal[SC_FXX]; part[s*n + i] = the
 // FP64 sum of the products' rounding errors.  Two rows per thread as in
-// k_gemv_part.
+// k_gemv_part; one = 1.0 and nz = -0.0 (products and sums as fused
+// multiply-adds, which the FP64 pipe that bounds this issues faster).
 __global__ void __launch_bounds__(MV_THREADS)
     k_gemv_part_fx(int64_t n, const double *__restrict__ A, int64_t lda,
-                   const double *__restrict__ v, const double *__restrict__ scal,
-                   unsigned long long *__restrict__ fx, double *__restrict__ part,
+                   const double *__restrict__ v, const double *__restrict__ scal, double one,
+                   double nz, unsigned long long *__restrict__ fx, double *__restrict__ part,
                    int64_t cols_per_split)
 {
     const int64_t i = ((int64_t)blockIdx.x * MV_THREADS + threadIdx.x) * 2;
@@ -283,9 +339,9 @@ __global__ void __launch_bounds__(MV_THREADS)
     for (int64_t j = j0; j < j1; ++j) {
         const double2 x = __ldg(reinterpret_cast<const double2 *>(a + j * lda));
         const double vj = __ldg(&v[j]);
-        const double p0 = __dmul_rn(x.x, vj), p1 = __dmul_rn(x.y, vj);
-        e0 = __dadd_rn(e0, __fma_rn(x.x, vj, -p0));
-        e1 = __dadd_rn(e1, __fma_rn(x.y, vj, -p1));
+        const double p0 = __fma_rn(x.x, vj, nz), p1 = __fma_rn(x.y, vj, nz);
+        e0 = __fma_rn(__fma_rn(x.x, vj, -p0), one, e0);
+        e1 = __fma_rn(__fma_rn(x.y, vj, -p1), one, e1);
         fx_add(s0, p0, c);
         fx_add(s1, p1, c);
     }
@@ -302,23 +358,46 @@ __global__ void __launch_bounds__(MV_THREADS)
     }
 }
 
-// out[i] = b[i] - (sum_s fx + sum_s part), the integer sums exact, rounded once
-__global__ void k_gemv_finish_fx(int64_t n, const unsigned long long *__restrict__ fx,
-                                 const double *__restrict__ part, int splits,
-                                 const double *__restrict__ scal, const double *__restrict__ b,
-                                 double *__restrict__ out)
+// out[i] = b[i] - (sum_s fx + sum_s part), the integer sums exact, rounded
+// once; *rn (zero before) = max |out[i]|.  A block takes 32 rows, its eight
+// warps the splits w, w + 8, ...: with one thread a row the chain of up to 64
+// dependent loads took 40 to 75 us.
+constexpr int FXF_WARPS = 8;
+__global__ void __launch_bounds__(32 * FXF_WARPS)
+    k_gemv_finish_fx(int64_t n, const unsigned long long *__restrict__ fx,
+                     const double *__restrict__ part, int splits, const double *__restrict__ scal,
+                     const double *__restrict__ b, double *__restrict__ out, double *rn)
 {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const int c = fx_anchor(scal[SC_FXA], scal[SC_FXX]);
+    __shared__ Fx192 sS[FXF_WARPS][32];
+    __shared__ double sE[FXF_WARPS][32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int64_t i = (int64_t)blockIdx.x * 32 + lane;
     Fx192 S{0, 0, 0};
     double es = 0.0;
-    for (int k = 0; k < splits; ++k) {
-        const unsigned long long *f = fx + (int64_t)k * 3 * n;
-        fx_merge(S, Fx192{f[i], f[n + i], f[2 * n + i]});
-        es = __dadd_rn(es, part[k * n + i]);
+    if (i < n) {
+#pragma unroll 4
+        for (int k = w; k < splits; k += FXF_WARPS) {
+            const unsigned long long *f = fx + (int64_t)k * 3 * n;
+            fx_merge(S, Fx192{f[i], f[n + i], f[2 * n + i]});
+            es = __dadd_rn(es, part[k * n + i]);
+        }
     }
-    out[i] = fx_residual(b[i], S, c, es);
+    sS[w][lane] = S;
+    sE[w][lane] = es;
+    __syncthreads();
+    if (w) return;
+    double r = 0.0;
+    if (i < n) {
+        for (int k = 1; k < FXF_WARPS; ++k) {
+            fx_merge(S, sS[k][lane]);
+            es = __dadd_rn(es, sE[k][lane]);
+        }
+        r = fx_residual(b[i], S, fx_anchor(scal[SC_FXA], scal[SC_FXX]), es);
+        out[i] = r;
+    }
+    r = fmax(0.0, fabs(r));  // (not a number counts as nothing)
+    for (int o = 16; o > 0; o >>= 1) r = fmax(r, __shfl_xor_sync(0xffffffffu, r, o));
+    if (lane == 0) atomic_max_nonneg(rn, r);
 }
 
 // out[i] = b[i] - sum_s part (b != NULL), or sum_s part
@@ -512,19 +591,19 @@ __global__ void __launch_bounds__(RED_THREADS)
     if (threadIdx.x == 0) scal[slot] = m;
 }
 
-// scal[slot] = max_i sum_s part[s*n + i] (||A||_inf from k_gemv_part<true>)
-__global__ void __launch_bounds__(RED_THREADS)
-    k_rowsum_max(int64_t n, const double *__restrict__ part, int splits, double *__restrict__ scal,
-                 int slot)
+// *an (zero before) = max_i sum_s part[s*n + i]: ||A||_inf from k_rowsums_part
+__global__ void __launch_bounds__(256)
+    k_rowsum_max(int64_t n, const double *__restrict__ part, int splits, double *an)
 {
-    double m = 0.0;
-    for (int64_t e = threadIdx.x; e < n; e += RED_THREADS) {
-        double s = 0.0;
-        for (int k = 0; k < splits; ++k) s += part[k * n + e];
-        m = fmax(m, s);
+    const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
+    double s = 0.0;
+    if (i < n) {
+#pragma unroll 8
+        for (int k = 0; k < splits; ++k) s += part[k * n + i];
     }
-    m = block_max(m);
-    if (threadIdx.x == 0) scal[slot] = m;
+    s = fmax(0.0, s);
+    for (int o = 16; o > 0; o >>= 1) s = fmax(s, __shfl_xor_sync(0xffffffffu, s, o));
+    if ((threadIdx.x & 31) == 0) atomic_max_nonneg(an, s);
 }
 
 // ---- host side ---------------------------------------------------------------
@@ -588,15 +667,29 @@ static void gemv(Ctx &c, const double *v, const double *b, double *out)
     const int64_t cps = ceil_div(c.n, c.splits64);
     dim3 grid((unsigned)ceil_div(c.n, 2 * MV_THREADS), (unsigned)c.splits64);
     c.tbeg(PH_GEMV);
-    k_gemv_part<false><<<grid, MV_THREADS, 0, c.stream>>>(c.n, c.d_A64, c.lda, v, c.d_part, cps);
+    k_gemv_part<<<grid, MV_THREADS, 0, c.stream>>>(c.n, c.d_A64, c.lda, v, c.d_part, cps);
     k_gemv_finish<<<(unsigned)ceil_div(c.n, 256), 256, 0, c.stream>>>(c.n, c.d_part, c.splits64, b,
                                                                       out);
     c.tend(PH_GEMV);
     c.launches += 2;
 }
 
+// scal[SC_FXA] = ||A||_inf, scal[SC_FXX] = ||x||_inf, scal[SC_BN] = ||b||_inf,
+// scal[SC_RN] = 0
+static void norms(Ctx &c, const double *x, const double *b)
+{
+    const int64_t cps = ceil_div(c.n, c.splits64);
+    dim3 grid((unsigned)ceil_div(c.n, 2 * MV_THREADS), (unsigned)c.splits64 + 1);
+    k_rowsums_part<<<grid, MV_THREADS, 0, c.stream>>>(c.n, c.d_A64, c.lda, 1.0, x, b, c.d_part, cps,
+                                                      c.d_scal);
+    k_rowsum_max<<<(unsigned)ceil_div(c.n, 256), 256, 0, c.stream>>>(c.n, c.d_part, c.splits64,
+                                                                     c.d_scal + SC_FXA);
+    c.launches += 2;
+}
+
 // r = b - A x with the FP64 matrix: to about u^2 (exact products, fx_add)
-// unless the context asks for a plain FP64 residual
+// unless the context asks for a plain FP64 residual.  The exact one leaves
+// ||A||_inf, ||x||_inf (its anchor), ||b||_inf and ||r||_inf in scal.
 static void residual(Ctx &c, const double *x, const double *b, double *r)
 {
     if (!c.residual_dd) {
@@ -606,16 +699,25 @@ static void residual(Ctx &c, const double *x, const double *b, double *r)
     const int64_t cps = ceil_div(c.n, c.splits64);
     dim3 grid((unsigned)ceil_div(c.n, 2 * MV_THREADS), (unsigned)c.splits64);
     c.tbeg(PH_GEMV);
-    // the anchor: ||A||_inf and ||x||_inf
-    k_gemv_part<true><<<grid, MV_THREADS, 0, c.stream>>>(c.n, c.d_A64, c.lda, nullptr, c.d_part, cps);
-    k_rowsum_max<<<1, RED_THREADS, 0, c.stream>>>(c.n, c.d_part, c.splits64, c.d_scal, SC_FXA);
-    k_nrm_inf<<<1, RED_THREADS, 0, c.stream>>>(c.n, x, c.d_scal, SC_FXX);
-    k_gemv_part_fx<<<grid, MV_THREADS, 0, c.stream>>>(c.n, c.d_A64, c.lda, x, c.d_scal,
+    norms(c, x, b);
+    k_gemv_part_fx<<<grid, MV_THREADS, 0, c.stream>>>(c.n, c.d_A64, c.lda, x, c.d_scal, 1.0, -0.0,
                                                       c.d_part_fx, c.d_part, cps);
-    k_gemv_finish_fx<<<(unsigned)ceil_div(c.n, 256), 256, 0, c.stream>>>(
-        c.n, c.d_part_fx, c.d_part, c.splits64, c.d_scal, b, r);
+    k_gemv_finish_fx<<<(unsigned)ceil_div(c.n, 32), 32 * FXF_WARPS, 0, c.stream>>>(
+        c.n, c.d_part_fx, c.d_part, c.splits64, c.d_scal, b, r, c.d_scal + SC_RN);
     c.tend(PH_GEMV);
-    c.launches += 5;
+    c.launches += 2;
+}
+
+// The residual and, in scal, the norms of the backward error: SC_RN, SC_BN
+// and ||A||_inf at SC_FXA.
+static void residual_and_norms(Ctx &c, const double *x, const double *b, double *r)
+{
+    if (!c.residual_dd) norms(c, x, b);
+    residual(c, x, b, r);
+    if (!c.residual_dd) {
+        k_nrm_inf<<<1, RED_THREADS, 0, c.stream>>>(c.n, r, c.d_scal, SC_RN);
+        c.launches += 1;
+    }
 }
 
 void enqueue_residual(Ctx &c, const double *x, const double *b, double *r) { residual(c, x, b, r); }
@@ -628,18 +730,20 @@ static double read_scalar(Ctx &c, int slot, cudaError_t *err)
     return v;
 }
 
+__global__ void k_copy_norms(const double *__restrict__ scal, double *__restrict__ out3)
+{
+    if (threadIdx.x == 0) {
+        out3[0] = scal[SC_RN];
+        out3[1] = scal[SC_FXA];
+        out3[2] = scal[SC_BN];
+    }
+}
+
 void enqueue_backward_error(Ctx &c, const double *b, const double *x, double *out3)
 {
-    residual(c, x, b, c.d_r);
-    k_nrm_inf<<<1, RED_THREADS, 0, c.stream>>>(c.n, c.d_r, out3, 0);
-    const int64_t cps = ceil_div(c.n, c.splits64);
-    dim3 grid((unsigned)ceil_div(c.n, 2 * MV_THREADS), (unsigned)c.splits64);
-    k_gemv_part<true><<<grid, MV_THREADS, 0, c.stream>>>(c.n, c.d_A64, c.lda, nullptr, c.d_part, cps);
-    k_gemv_finish<<<(unsigned)ceil_div(c.n, 256), 256, 0, c.stream>>>(c.n, c.d_part, c.splits64,
-                                                                      nullptr, c.d_w);
-    k_nrm_inf<<<1, RED_THREADS, 0, c.stream>>>(c.n, c.d_w, out3, 1);
-    k_nrm_inf<<<1, RED_THREADS, 0, c.stream>>>(c.n, b, out3, 2);
-    c.launches += 5;
+    residual_and_norms(c, x, b, c.d_r);
+    k_copy_norms<<<1, 32, 0, c.stream>>>(c.d_scal, out3);
+    c.launches += 1;
 }
 
 cudaError_t choose_start(Ctx &c, const double *b, const double *xp, double *xc, double *x0,
@@ -713,7 +817,6 @@ nrs_status run_gmres_ir(Ctx &c, const double *b, double *x, const double *x0, nr
     bool converged = false;
     double *h1 = c.d_scal + SC_COUNT;
     double *h2 = h1 + (m + 1);
-    bool have_an = false;
     for (outer = 0; outer < c.max_outer; ++outer) {
         residual(c, x, b, c.d_r);  // r = b - A x
         if (outer > 0) {
@@ -722,24 +825,16 @@ nrs_status run_gmres_ir(Ctx &c, const double *b, double *x, const double *x0, nr
             const double stag = read_scalar(c, SC_STAG, &e);
             if (e != cudaSuccess) CKE(e);
             if (stag != 0.0) {
-                k_nrm_inf<<<1, RED_THREADS, 0, c.stream>>>(n, c.d_r, c.d_scal, SC_RN);
-                k_nrm_inf<<<1, RED_THREADS, 0, c.stream>>>(n, b, c.d_scal, SC_BN);
-                c.launches += 2;
-                if (!have_an) {
-                    const int64_t cps = ceil_div(c.n, c.splits64);
-                    dim3 grid((unsigned)ceil_div(c.n, 2 * MV_THREADS), (unsigned)c.splits64);
-                    k_gemv_part<true><<<grid, MV_THREADS, 0, c.stream>>>(c.n, c.d_A64, c.lda,
-                                                                         nullptr, c.d_part, cps);
-                    k_gemv_finish<<<(unsigned)ceil_div(c.n, 256), 256, 0, c.stream>>>(
-                        c.n, c.d_part, c.splits64, nullptr, c.d_w);
-                    k_nrm_inf<<<1, RED_THREADS, 0, c.stream>>>(n, c.d_w, c.d_scal, SC_AN);
-                    c.launches += 3;
-                    have_an = true;
+                // the exact residual has left its norms in scal
+                if (!c.residual_dd) {
+                    norms(c, x, b);
+                    k_nrm_inf<<<1, RED_THREADS, 0, c.stream>>>(n, c.d_r, c.d_scal, SC_RN);
+                    c.launches += 1;
                 }
                 double sc[SC_COUNT];
                 CKE(cudaMemcpyAsync(sc, c.d_scal, sizeof(sc), cudaMemcpyDeviceToHost, c.stream));
                 CKE(cudaStreamSynchronize(c.stream));
-                if (sc[SC_RN] <= 1e-15 * (sc[SC_AN] * sc[SC_XN] + sc[SC_BN])) {
+                if (sc[SC_RN] <= 1e-15 * (sc[SC_FXA] * sc[SC_XN] + sc[SC_BN])) {
                     converged = true;
                     break;
                 }
@@ -806,7 +901,6 @@ static nrs_status finish_solve(Ctx &c, const double *b, double *x, nrs_solve_rep
                                int *inner_out, int outer, int inner_total, bool converged,
                                const double *dn_xn)
 {
-    const int64_t n = c.n;
     cudaError_t e = cudaSuccess;
     c.solves += 1;
     c.outer_total += outer;
@@ -826,18 +920,7 @@ static nrs_status finish_solve(Ctx &c, const double *b, double *x, nrs_solve_rep
     if (inner_out) *inner_out = inner_total;
     if (rep) {
         // backward error ||b - A x||_inf / (||A||_inf ||x||_inf + ||b||_inf)
-        residual(c, x, b, c.d_r);
-        k_nrm_inf<<<1, RED_THREADS, 0, c.stream>>>(n, c.d_r, c.d_scal, SC_RN);
-        k_nrm_inf<<<1, RED_THREADS, 0, c.stream>>>(n, b, c.d_scal, SC_BN);
-        {
-            const int64_t cps = ceil_div(c.n, c.splits64);
-            dim3 grid((unsigned)ceil_div(c.n, 2 * MV_THREADS), (unsigned)c.splits64);
-            k_gemv_part<true><<<grid, MV_THREADS, 0, c.stream>>>(c.n, c.d_A64, c.lda, nullptr,
-                                                                 c.d_part, cps);
-            k_gemv_finish<<<(unsigned)ceil_div(c.n, 256), 256, 0, c.stream>>>(
-                c.n, c.d_part, c.splits64, nullptr, c.d_w);
-            k_nrm_inf<<<1, RED_THREADS, 0, c.stream>>>(n, c.d_w, c.d_scal, SC_AN);
-        }
+        residual_and_norms(c, x, b, c.d_r);
         double sc[SC_COUNT];
         CKE(cudaMemcpyAsync(sc, c.d_scal, sizeof(sc), cudaMemcpyDeviceToHost, c.stream));
         CKE(cudaStreamSynchronize(c.stream));
@@ -845,7 +928,7 @@ static nrs_status finish_solve(Ctx &c, const double *b, double *x, nrs_solve_rep
         rep->inner = inner_total;
         rep->converged = converged ? 1 : 0;
         const double dn = dn_xn ? dn_xn[0] : sc[SC_DN], xn = dn_xn ? dn_xn[1] : sc[SC_XN];
-        rep->backward_err = sc[SC_RN] / (sc[SC_AN] * xn + sc[SC_BN]);
+        rep->backward_err = sc[SC_RN] / (sc[SC_FXA] * xn + sc[SC_BN]);
         rep->last_update = xn > 0 ? dn / xn : 0.0;
         rep->status = NRS_OK;
     }

@@ -244,6 +244,12 @@ nrs_status do_segments_and_assemble(Ctx *c, const D4 *x_lab, const D4 *Xw_lab, b
         // the FP32 copy first, alone on the GPU, so the factorisation can start;
         // then the FP64 matrix on the side stream beside the factorisation,
         // joined before the refinement uses it
+        if (!wait64 && x_lab != c->d_x) {
+            // the side stream reads the force points after the caller's stream has
+            // moved on, when the caller's buffer may hold something else
+            CK(cudaMemcpyAsync(c->d_x, x_lab, sizeof(D4) * c->N, cudaMemcpyDeviceToDevice, c->stream));
+            x_lab = c->d_x;
+        }
         nrs::launch_assemble32(*c, x_lab, a32, c->lda);
         if (wait64) {
             nrs::launch_assemble(*c, x_lab, c->d_A64, nullptr, c->lda, nullptr, from_state);

@@ -56,3 +56,26 @@ def test_matrix_bits_at_the_limits(N, Q, kind):
     got = ctx.assemble(xd, Xd).cpu().numpy().T
     want = O.assemble_stokeslet(x, X, nn.cpu().numpy(), eps, 1.0)
     assert np.array_equal(got, want)
+
+
+def test_the_callers_points_may_be_overwritten_in_stream_order():
+    # the FP64 matrix is assembled beside the caller's stream: what that does to
+    # its buffers after nrs_assemble must not reach it
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2001_06468_gb300 import nrs
+    N, Q = 1500, 15000
+    x, X, eps = _cloud("plain", N, Q, np.random.default_rng(12))
+    v = torch.from_numpy(np.random.default_rng(13).normal(size=3 * N)).cuda()
+    b = torch.zeros_like(v)
+    got = []
+    for overwrite in (False, True):
+        ctx = nrs.Context([0, N], [0, Q], [nrs.PRESCRIBED], eps=eps, factor_prec="tf32")
+        xd, Xd = torch.from_numpy(x).cuda(), torch.from_numpy(X).cuda()
+        ctx.nearest_build(xd, Xd)
+        ctx.assemble(xd, Xd, want_matrix=False)
+        if overwrite:
+            xd.zero_()
+            Xd.zero_()
+        got.append(ctx.residual(b, v).cpu().numpy())
+    assert np.array_equal(got[0], got[1])

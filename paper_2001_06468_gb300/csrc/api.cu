@@ -79,7 +79,6 @@ nrs_status alloc_all(Ctx *c)
         {(void **)&c->d_A64, sizeof(double) * lda * n},
         {(void **)&c->d_A32, sizeof(float) * lda * n},
         {(void **)&c->d_rowperm, sizeof(int32_t) * n},
-        {(void **)&c->d_lperm, sizeof(int32_t) * 64},
         {(void **)&c->d_gj_dinv, sizeof(float) * 2 * 64 * 64},
         {(void **)&c->d_gj_rt, sizeof(float) * 4 * 64 * lda},
         {(void **)&c->d_gj_cb, sizeof(float) * 4 * 64 * lda},
@@ -134,13 +133,13 @@ void free_all(Ctx *c)
                     c->d_x,      c->d_Xw,     c->d_b,      c->d_sol,        c->d_nn,
                     c->d_seg_ptr, c->d_perm,  c->d_cursor, c->d_Xs,         c->d_W,
                     c->d_R,      c->d_A64,    c->d_A32,    c->d_LU64,       c->d_rowperm,
-                    c->d_lperm,  c->d_info,   c->d_r,      c->d_xk,         c->d_w,
+                    c->d_info,   c->d_r,      c->d_xk,         c->d_w,
                     c->d_V,      c->d_H,      c->d_gv,     c->d_scal,       c->d_part,
                     c->d_t32,    c->d_t64,    c->d_flags,  c->d_status,     c->d_gj_dinv,
                     c->d_gj_rt,  c->d_gj_cb,  c->d_dpart,  c->d_bar,        c->d_pg_stats,
                     c->d_step_stats, c->d_Xsh, c->d_Xsl, c->d_xh, c->d_xl, c->d_gj_stage, c->d_gj_sync, c->d_part32,
                     c->d_part_fx, c->d_vf, c->d_gj2, c->d_gj2_r,
-                    c->d_vf2, c->d_Adf, c->d_asm_claim, c->d_nn_box};
+                    c->d_vf2, c->d_Adf, c->d_asm_claim, c->d_nn_box, c->d_LUinv};
     for (void *p : ptrs)
         if (p) cudaFree(p);
     void *tr[] = {c->d_tr, c->d_tr_save, c->d_tr_u, c->d_tr_part, c->d_vel_part, c->d_dp_K,
@@ -205,11 +204,17 @@ nrs_status do_factor(Ctx *c, int prec)
                 return fail(c, NRS_ENOMEM, "FP64 factor workspace does not fit");
             }
         }
+        if (!c->d_LUinv && dalloc(&c->d_LUinv, nrs::lu_inverse_doubles(c->n)) != cudaSuccess) {
+            cudaGetLastError();
+            c->d_LUinv = nullptr;
+            return fail(c, NRS_ENOMEM, "FP64 factor workspace does not fit");
+        }
         c->tbeg(nrs::PH_CONVERT);
         CK(cudaMemcpyAsync(c->d_LU64, c->d_A64, sizeof(double) * elems, cudaMemcpyDeviceToDevice,
                            c->stream));
         c->tend(nrs::PH_CONVERT);
-        nrs::run_lu_fp64(*c, c->d_LU64, c->lda);
+        if (nrs::run_lu_fp64(*c, c->d_LU64, c->lda) != 0)
+            return fail(c, NRS_ECUDA, "nrs_factor: the FP64 factorisation could not be launched");
     } else {
         if (!c->a32_fresh) {
             nrs::join_assembly(*c);  // the conversion reads the FP64 matrix

@@ -102,6 +102,7 @@ void launch_dp_error(Ctx &c, double h, double rtol, double atol, double *err);
 
 // ---- factorisation (lu.cu) -------------------------------------------------
 int run_lu_fp64(Ctx &c, double *A, int64_t lda);
+size_t lu_inverse_doubles(int64_t n);  // workspace of its diagonal triangles' inverses
 int run_gj_fp32(Ctx &c, float *M, int64_t lda, int prec);
 
 // two-level Gauss-Jordan with rank-256 tensor-core updates (gj2.cu), used by
@@ -237,8 +238,8 @@ struct Ctx {
     bool have_static = false, static_cache_valid = false;
     float *d_A32 = nullptr;    // FP32 copy, factored in place for the FP32/TF32/BF16 paths
     double *d_LU64 = nullptr;  // FP64 factor (plain path)
+    double *d_LUinv = nullptr; //   inverses of its diagonal blocks' 32 x 32 triangles
     int32_t *d_rowperm = nullptr;  // row order after pivoting: position i holds original row
-    int32_t *d_lperm = nullptr;    // row exchange of the current diagonal block
     bool a32_fresh = false;        // d_A32 holds the last assembly (not yet factored)
     float *d_gj_dinv = nullptr;    // Gauss-Jordan workspaces: D^{-1} (64 x 64)
     float *d_gj_rt = nullptr;      //   scaled block row, transposed (2 buffers of n x 64, then their TF32 lo parts)

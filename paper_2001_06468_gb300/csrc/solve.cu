@@ -86,97 +86,107 @@ __device__ __forceinline__ bool wait_flag(const int32_t *flags, int64_t j, int32
     return !*s_abort;
 }
 
-// y = L^{-1} P b  (L unit lower, P from rowperm), b in FP64, y in T.
-template <typename T, int NB>
-__global__ void __launch_bounds__(NB)
-    k_trsv_lower(int64_t n, const T *__restrict__ LU, int64_t lda, const int32_t *__restrict__ rowperm,
-                 const double *__restrict__ b, T *y, int32_t *flags, int32_t epoch, int32_t *status)
+// The triangular solves run as a chain over the 64-row blocks, so what counts
+// is the time from one block's flag to the next: the entries left of the
+// diagonal block are in registers before the flag is awaited (thread: row
+// tid mod 64, 16 columns), and the diagonal block is solved with the inverses
+// of its 32 x 32 triangles (lu.cu), three 32 x 32 products by eight lanes a
+// row, instead of 64 dependent steps with a division each (446 and 1197 us a
+// solve for n = 2406 so).
+constexpr int TR_THREADS = 256, TR_HB = 32;
+
+// sum over the eight lanes of a row (fixed order, every lane gets it)
+__device__ __forceinline__ double row_sum8(double v)
 {
-    __shared__ T ys[NB];
-    __shared__ T sacc[NB];
-    __shared__ T Ld[NB][NB + 1];
-    __shared__ int s_abort;
-    const int tid = threadIdx.x;
-    const int64_t nblk = ceil_div(n, NB);
-    for (int64_t blk = blockIdx.x; blk < nblk; blk += gridDim.x) {
-        const int64_t r0 = blk * NB;
-        const int rows = (int)min((int64_t)NB, n - r0);
-        const bool act = tid < rows;
-        // the diagonal block does not depend on other blocks: stage it first
-        if (act)
-            for (int c = 0; c < rows; ++c) Ld[tid][c] = LU[r0 + tid + (r0 + c) * lda];
-        T acc = act ? (T)b[rowperm[r0 + tid]] : T(0);
-        for (int64_t j = 0; j < blk; ++j) {
-            if (!wait_flag(flags, j, epoch, status, &s_abort)) return;
-            ys[tid] = __ldcg(&y[j * NB + tid]);
-            __syncthreads();
-            if (act) {
-                const T *col = LU + r0 + tid + j * NB * lda;
-#pragma unroll 8
-                for (int c = 0; c < NB; ++c) acc -= col[c * lda] * ys[c];
-            }
-            __syncthreads();
-        }
-        sacc[tid] = acc;
-        __syncthreads();
-        for (int c = 0; c < rows; ++c) {
-            const T yc = sacc[c];
-            if (act && tid > c) sacc[tid] -= Ld[tid][c] * yc;
-            __syncthreads();
-        }
-        if (act) y[r0 + tid] = sacc[tid];
-        __syncthreads();
-        if (tid == 0) {
-            __threadfence();
-            st_release(&flags[blk], epoch);
-        }
-    }
+#pragma unroll
+    for (int o = 1; o < 8; o <<= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
 }
 
-// x = U^{-1} y (U upper with its diagonal); the published blocks of x are
-// kept in T (xw) for the other CTAs, and written to x in TO.
-template <typename T, int NB, typename TO>
-__global__ void __launch_bounds__(NB)
-    k_trsv_upper(int64_t n, const T *__restrict__ LU, int64_t lda, const T *__restrict__ y, T *xw,
-                 TO *__restrict__ x, int32_t *flags, int32_t epoch, int32_t *status)
+// y = T^{-1} a for a 64 x 64 triangle given by the inverses of its 32 x 32
+// diagonal triangles (i0, i1: lower or upper) and its off-diagonal square (w);
+// thread (r, g) = (tid / 8, tid mod 8) holds columns 4g..4g+3 of row r of each.
+// LOWER: y0 = i0 a0, y1 = i1 (a1 - w y0); else y1 = i1 a1, y0 = i0 (a0 - w y1).
+template <bool LOWER>
+__device__ __forceinline__ void tri_solve64(const double (*i0)[4], double *a, double *y)
 {
-    __shared__ T xs[NB];
-    __shared__ T sacc[NB];
-    __shared__ T xout[NB];
-    __shared__ T Ud[NB][NB + 1];
+    const int r = threadIdx.x >> 3, g = threadIdx.x & 7;
+    const int first = LOWER ? 0 : TR_HB, second = TR_HB - first;
+    const double *mf = LOWER ? i0[0] : i0[1], *ms = LOWER ? i0[1] : i0[0], *w = i0[2];
+    auto dot = [&](const double *m, const double *v) {
+        double s = 0.0;
+#pragma unroll
+        for (int c = 0; c < 4; ++c) s = fma(m[c], v[4 * g + c], s);
+        return row_sum8(s);
+    };
+    const double u = dot(mf, a + first);
+    if (g == 0) y[first + r] = u;
+    __syncthreads();
+    const double t = a[second + r] - dot(w, y + first);
+    __syncthreads();  // a is read
+    if (g == 0) a[second + r] = t;
+    __syncthreads();
+    const double v = dot(ms, a + second);
+    if (g == 0) y[second + r] = v;
+    __syncthreads();
+}
+
+// LOWER: y = L^{-1} P b (L unit lower, P from rowperm); else y = U^{-1} b.
+// inv: the inverses of the diagonal blocks' triangles (lu.cu).  y is published
+// block by block; out (or NULL) receives a copy.
+template <bool LOWER>
+__global__ void __launch_bounds__(TR_THREADS)
+    k_trsv(int64_t n, const double *__restrict__ LU, int64_t lda, const double *__restrict__ inv,
+           const int32_t *__restrict__ rowperm, const double *__restrict__ b, double *y, double *out,
+           int32_t *flags, int32_t epoch, int32_t *status)
+{
+    __shared__ double ys[TR_NB], as[TR_NB], acc4[4][TR_NB];
     __shared__ int s_abort;
-    const int tid = threadIdx.x;
-    const int64_t nblk = ceil_div(n, NB);
+    const int tid = threadIdx.x, row = tid & 63, part = tid >> 6;
+    const int r = tid >> 3, g = tid & 7;
+    const int64_t nblk = ceil_div(n, TR_NB);
     for (int64_t i = blockIdx.x; i < nblk; i += gridDim.x) {
-        const int64_t blk = nblk - 1 - i;
-        const int64_t r0 = blk * NB;
-        const int rows = (int)min((int64_t)NB, n - r0);
-        const bool act = tid < rows;
-        if (act)
-            for (int c = 0; c < rows; ++c) Ud[tid][c] = LU[r0 + tid + (r0 + c) * lda];
-        T acc = act ? y[r0 + tid] : T(0);
-        for (int64_t j = nblk - 1; j > blk; --j) {
-            if (!wait_flag(flags, j, epoch, status, &s_abort)) return;
-            const int cols = (int)min((int64_t)NB, n - j * NB);
-            xs[tid] = tid < cols ? __ldcg(&xw[j * NB + tid]) : T(0);
-            __syncthreads();
-            if (act) {
-                const T *col = LU + r0 + tid + j * NB * lda;
-                for (int c = 0; c < cols; ++c) acc -= col[c * lda] * xs[c];
+        const int64_t blk = LOWER ? i : nblk - 1 - i;
+        const int64_t r0 = blk * TR_NB;
+        // this thread's share of the diagonal block (it depends on no other block)
+        double m[3][4];
+        {
+            const double *bi = inv + blk * 4 * TR_HB * TR_HB + (LOWER ? 0 : 2) * TR_HB * TR_HB;
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                m[0][c] = bi[r * TR_HB + 4 * g + c];
+                m[1][c] = bi[TR_HB * TR_HB + r * TR_HB + 4 * g + c];
+                const int64_t wr = r0 + (LOWER ? TR_HB : 0) + r;
+                const int64_t wc = r0 + (LOWER ? 0 : TR_HB) + 4 * g + c;
+                m[2][c] = wr < n && wc < n ? LU[wr + wc * lda] : 0.0;
             }
-            __syncthreads();
         }
-        sacc[tid] = acc;
+        const bool act = r0 + row < n;
+        double acc = 0.0;
+        if (part == 0 && act) acc = b[LOWER ? (int64_t)rowperm[r0 + row] : r0 + row];
+        const int64_t steps = LOWER ? blk : nblk - 1 - blk;
+        for (int64_t s = 0; s < steps; ++s) {
+            const int64_t j = LOWER ? s : nblk - 1 - s;
+            double v[16];
+#pragma unroll
+            for (int c = 0; c < 16; ++c) {
+                const int64_t col = j * TR_NB + 16 * part + c;
+                v[c] = act && col < n ? LU[r0 + row + col * lda] : 0.0;
+            }
+            if (!wait_flag(flags, j, epoch, status, &s_abort)) return;
+            if (tid < TR_NB) ys[tid] = j * TR_NB + tid < n ? __ldcg(&y[j * TR_NB + tid]) : 0.0;
+            __syncthreads();
+#pragma unroll
+            for (int c = 0; c < 16; ++c) acc = fma(-v[c], ys[16 * part + c], acc);
+        }
+        acc4[part][row] = acc;
         __syncthreads();
-        for (int c = rows - 1; c >= 0; --c) {
-            const T xc = sacc[c] / Ud[c][c];
-            if (act && tid < c) sacc[tid] -= Ud[tid][c] * xc;
-            if (tid == c) xout[c] = xc;
-            __syncthreads();
-        }
-        if (act) {
-            xw[r0 + tid] = xout[tid];
-            x[r0 + tid] = (TO)xout[tid];
+        if (tid < TR_NB) as[tid] = (acc4[0][tid] + acc4[1][tid]) + (acc4[2][tid] + acc4[3][tid]);
+        __syncthreads();
+        tri_solve64<LOWER>(m, as, ys);
+        if (tid < TR_NB && r0 + tid < n) {
+            y[r0 + tid] = ys[tid];
+            if (out) out[r0 + tid] = ys[tid];
         }
         __syncthreads();
         if (tid == 0) {
@@ -644,21 +654,22 @@ static cudaError_t apply_precond_impl(Ctx &c, const double *v, double *x)
         return cudaGetLastError();
     }
     {
-        auto kl = k_trsv_lower<double, TR_NB>;
-        auto ku = k_trsv_upper<double, TR_NB, double>;
+        auto kl = k_trsv<true>, ku = k_trsv<false>;
         int epoch = ++c.trsv_epoch;
         int64_t n = c.n, lda = c.lda;
-        double *LU = c.d_LU64;
+        double *LU = c.d_LU64, *inv = c.d_LUinv, *none = nullptr;
         double *y = c.d_t64;
-        void *args_l[] = {&n, &LU, &lda, &c.d_rowperm, &v, &y, &c.d_flags, &epoch, &c.d_status};
-        e = cudaLaunchCooperativeKernel((void *)kl, coop_grid(c, kl, TR_NB, nblk), TR_NB, args_l, 0,
-                                        c.stream);
+        void *args_l[] = {&n, &LU, &lda, &inv, &c.d_rowperm, &v, &y, &none, &c.d_flags, &epoch,
+                          &c.d_status};
+        e = cudaLaunchCooperativeKernel((void *)kl, coop_grid(c, kl, TR_THREADS, nblk), TR_THREADS,
+                                        args_l, 0, c.stream);
         if (e != cudaSuccess) return e;
         int epoch2 = ++c.trsv_epoch;
         double *xw = c.d_t64 + c.lda;  // second half of the FP64 work vector
-        void *args_u[] = {&n, &LU, &lda, &y, &xw, &x, &c.d_flags, &epoch2, &c.d_status};
-        return cudaLaunchCooperativeKernel((void *)ku, coop_grid(c, ku, TR_NB, nblk), TR_NB, args_u,
-                                           0, c.stream);
+        void *args_u[] = {&n, &LU, &lda, &inv, &c.d_rowperm, &y, &xw, &x, &c.d_flags, &epoch2,
+                          &c.d_status};
+        return cudaLaunchCooperativeKernel((void *)ku, coop_grid(c, ku, TR_THREADS, nblk),
+                                           TR_THREADS, args_u, 0, c.stream);
     }
 }
 

@@ -308,6 +308,7 @@ __device__ __forceinline__ double residual_fx_at(const PgArgs &a, double be, int
 {
     Fx192 S{0, 0, 0};
     double es = 0.0;
+#pragma unroll 4
     for (int k = 0; k < a.s64; ++k) {
         const unsigned long long *f = a.part_fx + (int64_t)k * 3 * a.n;
         fx_merge(S, Fx192{__ldcg(f + e), __ldcg(f + a.n + e), __ldcg(f + 2 * a.n + e)});
@@ -366,6 +367,7 @@ __device__ void mv32_partial(const PgArgs &a, double *sm)
 __device__ __forceinline__ double sum_parts(const PgArgs &a, int splits, int64_t e)
 {
     double s = 0.0;
+#pragma unroll 8
     for (int k = 0; k < splits; ++k) s += __ldcg(a.part + k * a.n + e);
     return s;
 }
@@ -373,6 +375,7 @@ __device__ __forceinline__ double sum_parts(const PgArgs &a, int splits, int64_t
 __device__ __forceinline__ double sum_parts32(const PgArgs &a, int64_t e)
 {
     double s = 0.0;
+#pragma unroll 8
     for (int k = 0; k < a.s32; ++k) s += __ldcg(a.part32 + k * a.n + e);
     return s;
 }
@@ -515,25 +518,25 @@ __global__ void __launch_bounds__(PG_THREADS, MINB) k_gmres_ir(PgArgs a)
     double *dp1 = a.dpart + (1 * PG_MAXCH + (int64_t)blockIdx.x) * (m + 2);
     double *dp2 = a.dpart + (2 * PG_MAXCH + (int64_t)blockIdx.x) * (m + 2);
 
-    if (a.cold) {  // x = M b
-        for (int64_t e = e0 + threadIdx.x; e < e1; e += PG_THREADS) a.vf[e] = df_split(__ldg(a.b + e));
-        if (!grid_sync(a, &s_ok, tgt)) return;
-        mv32_partial(a, smv);
-        if (!grid_sync(a, &s_ok, tgt)) return;
-        for (int64_t e = e0 + threadIdx.x; e < e1; e += PG_THREADS) a.x[e] = sum_parts32(a, e);
-        if (!grid_sync(a, &s_ok, tgt)) return;
-    }
     int outer = 0, inner_total = 0, converged = 0;
     double dn = 0.0, xn = 0.0, dn_prev = 0.0, normA = -1.0;
     bool stagnant = false;
-    if (a.dd) {
-        // the exact residual's anchor needs ||A||_inf and ||x||_inf up front
-        mv64_partial<true>(a, nullptr, 1.0, smv);
+    // x = M b (cold start); the exact residual's anchor needs ||A||_inf and
+    // ||x||_inf up front, and the row sums of |A| share the product's phase
+    if (a.cold) {
+        for (int64_t e = e0 + threadIdx.x; e < e1; e += PG_THREADS) a.vf[e] = df_split(__ldg(a.b + e));
+        if (!grid_sync(a, &s_ok, tgt)) return;
+        mv32_partial(a, smv);
+    }
+    if (a.dd) mv64_partial<true>(a, nullptr, 1.0, smv);
+    if (a.cold || a.dd) {
         if (!grid_sync(a, &s_ok, tgt)) return;
         double amax = 0.0, xmax = 0.0;
         for (int64_t e = e0 + threadIdx.x; e < e1; e += PG_THREADS) {
-            amax = fmax(amax, sum_parts(a, a.s64, e));
-            xmax = fmax(xmax, fabs(__ldcg(a.x + e)));
+            const double xe = a.cold ? sum_parts32(a, e) : __ldcg(a.x + e);
+            if (a.cold) a.x[e] = xe;
+            if (a.dd) amax = fmax(amax, sum_parts(a, a.s64, e));
+            xmax = fmax(xmax, fabs(xe));
         }
         amax = block_max_all(amax, sred);
         xmax = block_max_all(xmax, sred);
@@ -542,8 +545,10 @@ __global__ void __launch_bounds__(PG_THREADS, MINB) k_gmres_ir(PgArgs a)
             dp0[1] = xmax;
         }
         if (!grid_sync(a, &s_ok, tgt)) return;
-        normA = chunk_total(a, 1, 2, true, sred);
-        xn = chunk_total(a, 0, 1, true, sred);
+        if (a.dd) {
+            normA = chunk_total(a, 1, 2, true, sred);
+            xn = chunk_total(a, 0, 1, true, sred);
+        }
     }
     double eta_prev = INFINITY;  // backward error of the previous step's residual
     int n_exact = 0, n_work = 0;  // residuals formed: exact (or FP64), working precision
@@ -832,15 +837,20 @@ int pg_max_coresident(const Ctx &c)
 
 size_t pg_dpart_doubles(int max_inner) { return (size_t)3 * PG_MAXCH * (max_inner + 2); }
 
-// The number of column splits s in [lo, 64] of a product with rc row tiles on a
-// grid of G CTAs: the smallest whose rc s tiles fill their last wave to 97 %,
-// else the best fill.
-static int pick_splits(int64_t rc, int G, int lo)
+// The number of column splits of a product of n columns with rc row tiles on
+// a grid of G CTAs: from lo on, and from as many as fit one wave, the smallest
+// whose rc s tiles fill their last wave to 97 %, else the best fill.  Every
+// element of the product is the sum of s partial sums, read one after the
+// other, so a split keeps at least PG_MIN_COLS columns (n = 288 on 152 CTAs
+// had taken 60 splits: 187 us a solve; 142 with 9 and two barriers fewer).
+constexpr int PG_MIN_COLS = 32;
+static int pick_splits(int64_t n, int64_t rc, int G, int lo)
 {
-    lo = std::max(1, std::min(lo, 64));
+    const int hi = (int)std::max<int64_t>(lo, std::min<int64_t>(64, n / PG_MIN_COLS));
+    lo = std::max(lo, std::min(hi, (int)(G / rc)));
     int best = lo;
     double best_fill = -1.0;
-    for (int s = lo; s <= 64; ++s) {
+    for (int s = lo; s <= hi; ++s) {
         const int64_t t = rc * s;
         const double fill = (double)t / (double)(ceil_div(t, G) * G);
         if (fill > best_fill + 1e-12) {
@@ -886,13 +896,12 @@ cudaError_t launch_gmres_persistent(Ctx &c, const double *b, double *x, bool col
     a.cold = cold ? 1 : 0;
     a.rc64 = (int)ceil_div(c.n, MV64_ROWS);
     a.rc32 = (int)ceil_div(c.n, MV32_ROWS);
-    // column splits: at least one tile per CTA, then the fewest splits whose
-    // tiles fill the last wave of the grid to 97 % (at n = 27648: 432 row
-    // tiles on 304 CTAs fill 71 % with one split, 99.5 % with seven)
-    a.s64 = pick_splits(a.rc64, G, (int)std::max<int64_t>(1, ceil_div(G, a.rc64)));
-    // at least 8 column splits for the FP32 product: each partial sum then
-    // covers at most n / 8 columns before the splits are added in FP64
-    a.s32 = pick_splits(a.rc32, G, (int)std::max<int64_t>(8, ceil_div(G, a.rc32)));
+    // column splits (at n = 27648: 432 row tiles on 304 CTAs fill 71 % of the
+    // last wave with one split, 99.5 % with seven); at least 8 for the FP32
+    // product: each partial sum then covers at most n / 8 columns before the
+    // splits are added in FP64
+    a.s64 = pick_splits(c.n, a.rc64, G, 1);
+    a.s32 = pick_splits(c.n, a.rc32, G, 8);
     a.s64 = (int)std::min<int64_t>(a.s64, c.n);
     a.s32 = (int)std::min<int64_t>(a.s32, c.n);
     a.cps64 = ceil_div(c.n, a.s64);

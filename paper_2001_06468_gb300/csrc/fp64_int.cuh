@@ -250,4 +250,78 @@ NRS_HD bool split_pair(double v, float &hi, float &lo)
     return true;
 }
 
+// ---- exact products placed in a 192-bit integer (the exact residual) ----------
+// A double as the factor of many products: |v| = m 2^(max(ex, 1) - 1075) with
+// ex its exponent field, and s = max(ex, 1) - 1075 - c the part of the
+// product's place that it settles; f: its high word.
+struct FxFactor {
+    uint64_t m;
+    int32_t s;
+    uint32_t f;
+};
+
+// |x v| 2^-L in three words, little-endian
+struct FxPlaced {
+    uint64_t z0, z1, z2;
+};
+
+NRS_HD FxFactor fx_factor(double v, int c)
+{
+    const uint64_t u = double_bits(v);
+    const uint32_t ex = (hi32(u) >> 20) & 0x7ffu, e1 = ex > 1u ? ex : 1u;
+    return FxFactor{(u & 0xfffffffffffffULL) | ((uint64_t)(ex < 1u ? ex : 1u) << 52),
+                    (int32_t)e1 - 1075 - c, hi32(u)};
+}
+
+// a 106-bit product
+struct FxWords {
+    uint32_t w0, w1, w2, w3;
+};
+
+NRS_HD FxWords fx_product(uint64_t x, uint64_t v)
+{
+    const uint64_t p = wide(lo32(x), lo32(v), 0);
+    const uint64_t q = wide(lo32(x), hi32(v), hi32(p));
+    const uint64_t r = wide(hi32(x), lo32(v), lo32(q));
+    const uint64_t t = wide(hi32(x), hi32(v), (uint64_t)hi32(q) + hi32(r));
+    return FxWords{lo32(p), lo32(r), lo32(t), hi32(t)};
+}
+
+// A product whose place s is outside [0, 86], moved so that it is inside: down,
+// dropping what falls below bit 0, or (a short product, of a subnormal factor)
+// up.  False if it has no room.
+NRS_HD bool fx_move(FxWords &w, int32_t &s)
+{
+    if ((w.w0 | w.w1 | w.w2 | w.w3) == 0) s = 0;
+    if (s < -127) w = FxWords{0, 0, 0, 0}, s = 0;
+    while (s < 0) {
+        const uint32_t k = s < -31 ? 31u : (uint32_t)-s;
+        w = FxWords{funnel_l(w.w0, w.w1, 32u - k), funnel_l(w.w1, w.w2, 32u - k),
+                    funnel_l(w.w2, w.w3, 32u - k), w.w3 >> k};
+        s += (int32_t)k;
+    }
+    while (s > 86) {
+        if (w.w3 >> 9) return false;  // 106 bits already
+        w = FxWords{w.w0 << 1, funnel_l(w.w0, w.w1, 1), funnel_l(w.w1, w.w2, 1),
+                    funnel_l(w.w2, w.w3, 1)};
+        --s;
+    }
+    return true;
+}
+
+// The product placed s bits up, 0 <= s <= 86 (its 106 bits fit): five words of
+// 32 bits from a shift by s mod 32, moved up by s / 32 words.
+NRS_HD FxPlaced fx_place(const FxWords &w, uint32_t s)
+{
+    const uint32_t b = s & 31u;
+    const uint32_t y0 = w.w0 << b, y1 = funnel_l(w.w0, w.w1, b), y2 = funnel_l(w.w1, w.w2, b);
+    const uint32_t y3 = funnel_l(w.w2, w.w3, b), y4 = funnel_l(w.w3, 0u, b);
+    const bool q1 = s >= 32u, q2 = s >= 64u;
+    const uint32_t z0 = q1 ? 0u : y0, z1 = q1 ? (q2 ? 0u : y0) : y1;
+    const uint32_t z2 = q1 ? (q2 ? y0 : y1) : y2, z3 = q1 ? (q2 ? y1 : y2) : y3;
+    const uint32_t z4 = q1 ? (q2 ? y2 : y3) : y4, z5 = q1 ? (q2 ? y3 : y4) : 0u;
+    return FxPlaced{((uint64_t)z1 << 32) | z0, ((uint64_t)z3 << 32) | z2,
+                    ((uint64_t)z5 << 32) | z4};
+}
+
 }  // namespace nrs

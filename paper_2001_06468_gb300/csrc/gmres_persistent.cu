@@ -21,9 +21,8 @@
 //
 // The residual b - A x is computed to about u^2 by default (the
 // three-precision form of Carson & Higham, whose solution reaches working
-// accuracy for kappa(A) up to about 1/u) -- every product's rounded value
-// summed exactly as an integer, its rounding error in FP64 (fx_add) -- or in
-// FP64.
+// accuracy for kappa(A) up to about 1/u) -- the products summed exactly, as
+// integers (fx_madd) -- or in FP64.
 //
 // Stopping rule: that of k_outer_check (solve.cu), plus one for very
 // ill-conditioned systems, where an FP64 residual leaves corrections of about
@@ -232,11 +231,11 @@ __device__ void mv64df_partial(const PgArgs &a, double scale, double *sm)
     }
 }
 
-// The residual's product, exact: fx[s][.][i] = sum_{j in split s} fl(A[i, j]
-// v[j]) as a 192-bit integer (fx_add, anchor c) and part[s][i] = the FP64 sum
-// of the products' rounding errors; the tile layout of mv64_partial.  The 8
+// The residual's product, exact: fx[s][.][i] = sum_{j in split s} A[i, j] v[j]
+// as a 192-bit integer (fx_madd, anchor c) and part[s][i] = 0, or NaN
+// (fx_poison); the tile layout of mv64_partial.  The 8
 // column groups are merged by a tree in shared memory (groups g + h into g,
-// h = 4, 2, 1): exact for the integers, a fixed order for the error sums.
+// h = 4, 2, 1).
 __device__ void mv64fx_partial(const PgArgs &a, const double *v, int c, double *sm)
 {
     const int64_t tiles = (int64_t)a.rc64 * a.s64;
@@ -247,21 +246,20 @@ __device__ void mv64fx_partial(const PgArgs &a, const double *v, int c, double *
         const int64_t i = rc * MV64_ROWS + 2 * lane;
         const int64_t j0 = s * a.cps64, j1 = min(a.n, j0 + a.cps64);
         Fx192 s0{0, 0, 0}, s1{0, 0, 0};
-        double e0 = 0.0, e1 = 0.0;
+        uint32_t b0 = 0, b1 = 0, bv = 0;
         if (i < a.n) {
             const double *col = a.A + i;
 #pragma unroll 4
             for (int64_t j = j0 + grp; j < j1; j += MV_GROUPS) {
                 pf_line<8>(a.A, a.lda, a.n, rc * MV64_ROWS, j, j1, lane);
                 const double2 x = __ldg(reinterpret_cast<const double2 *>(col + j * a.lda));
-                const double vj = __ldcg(v + j);
-                const double p0 = __dmul_rn(x.x, vj), p1 = __dmul_rn(x.y, vj);
-                e0 = __dadd_rn(e0, __fma_rn(x.x, vj, -p0));
-                e1 = __dadd_rn(e1, __fma_rn(x.y, vj, -p1));
-                fx_add(s0, p0, c);
-                fx_add(s1, p1, c);
+                const FxFactor vj = fx_factor(__ldcg(v + j), c);
+                bv = max(bv, vj.f & 0x7fffffffu);
+                fx_madd(s0, b0, x.x, vj);
+                fx_madd(s1, b1, x.y, vj);
             }
         }
+        double e0 = fx_poison(max(b0, bv)), e1 = fx_poison(max(b1, bv));
         // tree over the column groups: slot k holds rows 2l, 2l+1 of group
         // h + k as 8 values (3 + 3 integer words, 2 error sums)
         for (int h = MV_GROUPS / 2; h >= 1; h >>= 1) {

@@ -13,6 +13,7 @@
 #include <vector>
 
 #include "../../include/nrs.h"
+#include "fp64_int.cuh"
 
 namespace nrs {
 
@@ -384,25 +385,31 @@ __device__ __forceinline__ void dd_two_sum(double a, double b, double &s, double
 // residual precision of three-precision GMRES-IR).  Double-double sums cost 7
 // FP64 operations per matrix entry, and GB300 issues FP64 at about two lanes
 // per SM per clock, so they bound the product far above its memory time.
-// Here each product p = A_ij x_j is rounded in FP64 (one multiply), its
-// rounding error e = A_ij x_j - p taken exactly by one fused multiply-add, and
-// the errors summed in FP64 (one add): 3 FP64 operations.  The rounded
-// products themselves are added EXACTLY on the integer pipe to a 192-bit
-// two's-complement integer S standing for S 2^L.  The anchor L comes from a
+// Here each product A_ij x_j is formed exactly, 106 bits from the two 53-bit
+// significands, and added EXACTLY to a 192-bit two's-complement integer S
+// standing for S 2^L, all on the integer pipe (fp64_int.cuh): some 50
+// instructions of 2 clocks a warp.  (With the product and its rounding error
+// from the FP64 pipe, 64 clocks an operation, and only the sum in integers, an
+// entry took 192 clocks and more: six solves at n = 2592 with their reports 4.42
+// ms, now 4.21; a step at n = 14064 1.2 ms less.)  The anchor L
+// comes from a
 // bound on every partial sum, |sum_j A_ij x_j| <= ||A||_inf ||x||_inf < 2^E:
 // with L = E - 189 the sums never overflow (|S| < 2^191), and a product loses
 // less than 2^L (about 2^-187 ||A|| ||x||) when its bits below 2^L are
 // dropped.  Integer addition is associative, so splitting the sum over
 // threads, column groups and column splits changes nothing: the product's
 // integer part is exact and deterministic whatever the order.  A non-finite
-// product makes its FP64 error term NaN, so it still reaches the residual.
+// factor, or a product beyond the integer's range, makes the row's FP64 term
+// NaN, so it still reaches the residual.
+constexpr uint32_t kInfHigh = 0x7ff00000u;  // high word of infinity
+
 struct Fx192 {
     unsigned long long w0, w1, w2;  // little-endian 64-bit words
 };
 
 // c = 1075 + L for sums bounded by an * xn (an, xn >= 0).  When the bound is
-// zero every product is zero; when it is not finite, products overflow to
-// non-finite error terms; any anchor serves then (E = 0).
+// zero every product is zero; when it is not finite, some row is NaN whatever the
+// anchor; E = 0 then.
 __device__ __forceinline__ int fx_anchor(double an, double xn)
 {
     const bool ok = an > 0.0 && xn > 0.0 && isfinite(an) && isfinite(xn);
@@ -410,26 +417,23 @@ __device__ __forceinline__ int fx_anchor(double an, double xn)
     return 1075 + E - 189;
 }
 
-// S += p 2^-L exactly, truncated toward zero below bit 0 (c = 1075 + L).  The
-// double is m 2^(e - 1075) with m its 53-bit integer significand (no implicit
-// bit for subnormals, e raised to 1), so m lands at bit s = e - c of S; the
-// magnitude is placed in three words and added, or subtracted as its one's
-// complement with a carry in, by one chain of extended-precision adds.
-__device__ __forceinline__ void fx_add(Fx192 &a, double p, int c)
+// a += x v 2^-L exactly, truncated toward zero below bit 0: the magnitude is
+// placed in three words and added, or subtracted as its one's complement with a
+// carry in, by one chain of extended-precision adds.  big: the largest high
+// word of |x| so far, raised to infinity's when the product does not fit.
+__device__ __forceinline__ void fx_madd(Fx192 &a, uint32_t &big, double x, const FxFactor &v)
 {
-    const unsigned long long bits = (unsigned long long)__double_as_longlong(p);
-    const int ex = (int)(bits >> 52) & 0x7ff;
-    unsigned long long m = (bits & 0xfffffffffffffULL) | ((unsigned long long)(ex != 0) << 52);
-    int s = max(ex, 1) - c;
-    m >>= min(max(-s, 0), 63);  // the bits below 2^L
-    s = max(s, 0);
-    const int wi = s >> 6, b = s & 63;
-    const unsigned long long lo = m << b, hi = (m >> 1) >> (63 - b);
-    const unsigned long long neg = (unsigned long long)((long long)bits >> 63);
-    const unsigned long long x0 = (wi == 0 ? lo : 0ULL) ^ neg;
-    const unsigned long long x1 = (wi == 0 ? hi : (wi == 1 ? lo : 0ULL)) ^ neg;
-    const unsigned long long x2 = (wi == 1 ? hi : (wi == 2 ? lo : 0ULL)) ^ neg;
-    // carry in = 1 for negative p: neg + neg carries out exactly when neg != 0
+    const uint64_t u = double_bits(x);
+    const uint32_t h = hi32(u), ex = (h >> 20) & 0x7ffu;
+    big = max(big, h & 0x7fffffffu);
+    const uint64_t m = (u & 0xfffffffffffffULL) | ((uint64_t)min(ex, 1u) << 52);
+    int32_t s = (int32_t)max(ex, 1u) + v.s;
+    FxWords w = fx_product(m, v.m);
+    if ((uint32_t)s > 86u && !fx_move(w, s)) big = kInfHigh;
+    const FxPlaced z = fx_place(w, (uint32_t)s);
+    const unsigned long long neg = (unsigned long long)(long long)((int32_t)(h ^ v.f) >> 31);
+    const unsigned long long x0 = z.z0 ^ neg, x1 = z.z1 ^ neg, x2 = z.z2 ^ neg;
+    // carry in = 1 for a negative product: neg + neg carries out exactly when neg != 0
     asm("{\n\t.reg .u64 t;\n\t"
         "add.cc.u64 t, %3, %3;\n\t"
         "addc.cc.u64 %0, %0, %4;\n\t"
@@ -437,6 +441,12 @@ __device__ __forceinline__ void fx_add(Fx192 &a, double p, int c)
         "addc.u64 %2, %2, %6;\n\t}"
         : "+l"(a.w0), "+l"(a.w1), "+l"(a.w2)
         : "l"(neg), "l"(x0), "l"(x1), "l"(x2));
+}
+
+// What a row's residual adds in FP64: nothing, or NaN
+__device__ __forceinline__ double fx_poison(uint32_t big)
+{
+    return big >= kInfHigh ? __longlong_as_double(0x7ff8000000000000LL) : 0.0;
 }
 
 // a += b (exact, modulo 2^192)
@@ -485,8 +495,7 @@ __device__ __forceinline__ void fx_to_dd(Fx192 a, int c, double &hi, double &lo)
 }
 
 // b - (S 2^L + es) in double-double, rounded once: the residual of one row
-// from its exact integer product sum S and the FP64 sum es of the products'
-// rounding errors.
+// from its exact integer product sum S; es is 0, or NaN (fx_poison).
 __device__ __forceinline__ double fx_residual(double b, const Fx192 &S, int c, double es)
 {
     double h, l, s, e;

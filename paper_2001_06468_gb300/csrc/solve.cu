@@ -325,16 +325,14 @@ __global__ void __launch_bounds__(MV_THREADS)
     if (i + 3 < n) p[3] = (double)s3 + (double)c3;
 }
 
-// The residual's product, exact (fx_add): fx[(s*3 + w)*n + i] = word w of
-// sum_{j in split s} fl(A[i,j] v[j]) as a 192-bit integer with the anchor of
-// ||A||_inf = scal[SC_FXA], ||v||_inf = scal[SC_FXX]; part[s*n + i] = the
-// FP64 sum of the products' rounding errors.  Two rows per thread as in
-// k_gemv_part; one = 1.0 and nz = -0.0 (products and sums as fused
-// multiply-adds, which the FP64 pipe that bounds this issues faster).
+// The residual's product, exact (fx_madd): fx[(s*3 + w)*n + i] = word w of
+// sum_{j in split s} A[i,j] v[j] as a 192-bit integer with the anchor of
+// ||A||_inf = scal[SC_FXA], ||v||_inf = scal[SC_FXX]; part[s*n + i] = 0, or NaN
+// (fx_poison).  Two rows per thread as in k_gemv_part.
 __global__ void __launch_bounds__(MV_THREADS)
     k_gemv_part_fx(int64_t n, const double *__restrict__ A, int64_t lda,
-                   const double *__restrict__ v, const double *__restrict__ scal, double one,
-                   double nz, unsigned long long *__restrict__ fx, double *__restrict__ part,
+                   const double *__restrict__ v, const double *__restrict__ scal,
+                   unsigned long long *__restrict__ fx, double *__restrict__ part,
                    int64_t cols_per_split)
 {
     const int64_t i = ((int64_t)blockIdx.x * MV_THREADS + threadIdx.x) * 2;
@@ -343,18 +341,17 @@ __global__ void __launch_bounds__(MV_THREADS)
     if (i >= n) return;
     const int c = fx_anchor(scal[SC_FXA], scal[SC_FXX]);
     Fx192 s0{0, 0, 0}, s1{0, 0, 0};
-    double e0 = 0.0, e1 = 0.0;
+    uint32_t b0 = 0, b1 = 0, bv = 0;
     const double *a = A + i;
 #pragma unroll 4
     for (int64_t j = j0; j < j1; ++j) {
         const double2 x = __ldg(reinterpret_cast<const double2 *>(a + j * lda));
-        const double vj = __ldg(&v[j]);
-        const double p0 = __fma_rn(x.x, vj, nz), p1 = __fma_rn(x.y, vj, nz);
-        e0 = __fma_rn(__fma_rn(x.x, vj, -p0), one, e0);
-        e1 = __fma_rn(__fma_rn(x.y, vj, -p1), one, e1);
-        fx_add(s0, p0, c);
-        fx_add(s1, p1, c);
+        const FxFactor vj = fx_factor(__ldg(&v[j]), c);
+        bv = max(bv, vj.f & 0x7fffffffu);
+        fx_madd(s0, b0, x.x, vj);
+        fx_madd(s1, b1, x.y, vj);
     }
+    const double e0 = fx_poison(max(b0, bv)), e1 = fx_poison(max(b1, bv));
     unsigned long long *f = fx + blockIdx.y * 3 * n;
     f[i] = s0.w0;
     f[n + i] = s0.w1;
@@ -698,7 +695,7 @@ static void norms(Ctx &c, const double *x, const double *b)
     c.launches += 2;
 }
 
-// r = b - A x with the FP64 matrix: to about u^2 (exact products, fx_add)
+// r = b - A x with the FP64 matrix: to about u^2 (exact products, fx_madd)
 // unless the context asks for a plain FP64 residual.  The exact one leaves
 // ||A||_inf, ||x||_inf (its anchor), ||b||_inf and ||r||_inf in scal.
 static void residual(Ctx &c, const double *x, const double *b, double *r)
@@ -711,8 +708,8 @@ static void residual(Ctx &c, const double *x, const double *b, double *r)
     dim3 grid((unsigned)ceil_div(c.n, 2 * MV_THREADS), (unsigned)c.splits64);
     c.tbeg(PH_GEMV);
     norms(c, x, b);
-    k_gemv_part_fx<<<grid, MV_THREADS, 0, c.stream>>>(c.n, c.d_A64, c.lda, x, c.d_scal, 1.0, -0.0,
-                                                      c.d_part_fx, c.d_part, cps);
+    k_gemv_part_fx<<<grid, MV_THREADS, 0, c.stream>>>(c.n, c.d_A64, c.lda, x, c.d_scal, c.d_part_fx,
+                                                      c.d_part, cps);
     k_gemv_finish_fx<<<(unsigned)ceil_div(c.n, 32), 32 * FXF_WARPS, 0, c.stream>>>(
         c.n, c.d_part_fx, c.d_part, c.splits64, c.d_scal, b, r, c.d_scal + SC_RN);
     c.tend(PH_GEMV);

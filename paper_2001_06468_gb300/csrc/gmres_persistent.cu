@@ -54,7 +54,6 @@ struct PgArgs {
     const double *b;
     double *x;            // in: starting guess unless cold; out: solution
     double *V;            // Krylov basis, n x (m+1), leading dimension ldv
-    double *w;            // n: A v, then the residual
     double *part;         // partial sums of the FP64 products [splits][n]
     double *part32;       // partial sums of the FP32 products [splits][n]
     unsigned long long *part_fx;  // the exact residual's integer partial sums [splits][3][n]
@@ -322,7 +321,8 @@ __device__ __forceinline__ double residual_fx_at(const PgArgs &a, double be, int
 // kappa(A) u_fp32 >> 1, which FP32 products of a rounded v (2^-24) are not.
 // 128 rows per tile, lane l takes rows 4l..4l+3 (one 16-byte load per column);
 // the 8 column groups are added in FP64 in a fixed order.
-__device__ void mv32_partial(const PgArgs &a, double *sm)
+template <class Col>
+__device__ __forceinline__ void mv32_tiles(const PgArgs &a, double *sm, Col col)
 {
     const int64_t tiles = (int64_t)a.rc32 * a.s32;
     const int lane = threadIdx.x & 31, grp = threadIdx.x >> 5;
@@ -330,15 +330,16 @@ __device__ void mv32_partial(const PgArgs &a, double *sm)
         const int64_t rc = t % a.rc32, s = t / a.rc32;
         const int64_t i = rc * MV32_ROWS + 4 * lane;
         const int64_t j0 = s * a.cps32, j1 = min(a.n, j0 + a.cps32);
+        col.stage(j0, j1);
         float s0 = 0.0f, s1 = 0.0f, s2 = 0.0f, s3 = 0.0f;
         float c0 = 0.0f, c1 = 0.0f, c2 = 0.0f, c3 = 0.0f;
         if (i < a.n) {
-            const float *col = a.M + i;
+            const float *m = a.M + i;
 #pragma unroll 4
             for (int64_t j = j0 + grp; j < j1; j += MV_GROUPS) {
                 pf_line<4>(a.M, a.lda, a.n, rc * MV32_ROWS, j, j1, lane);
-                const float4 x = __ldg(reinterpret_cast<const float4 *>(col + j * a.lda));
-                const float2 vj = __ldcg(a.vf + j);
+                const float4 x = __ldg(reinterpret_cast<const float4 *>(m + j * a.lda));
+                const float2 vj = col.at(j);
                 df_fma(x.x, vj, s0, c0);
                 df_fma(x.y, vj, s1, c1);
                 df_fma(x.z, vj, s2, c2);
@@ -362,6 +363,18 @@ __device__ void mv32_partial(const PgArgs &a, double *sm)
     }
 }
 
+// the vector a.vf, written a phase before
+struct ColStored {
+    const float2 *vf;
+    __device__ __forceinline__ void stage(int64_t, int64_t) {}
+    __device__ __forceinline__ float2 at(int64_t j) const { return __ldcg(vf + j); }
+};
+
+__device__ __forceinline__ void mv32_partial(const PgArgs &a, double *sm)
+{
+    mv32_tiles(a, sm, ColStored{a.vf});
+}
+
 __device__ __forceinline__ double sum_parts(const PgArgs &a, int splits, int64_t e)
 {
     double s = 0.0;
@@ -376,6 +389,34 @@ __device__ __forceinline__ double sum_parts32(const PgArgs &a, int64_t e)
 #pragma unroll 8
     for (int k = 0; k < a.s32; ++k) s += __ldcg(a.part32 + k * a.n + e);
     return s;
+}
+
+// The vector formed by each CTA for the columns of its own tiles, from the
+// partial sums of the phase before: for a small system this costs less than the
+// grid barrier between forming a vector and multiplying it (a phase takes about
+// 5.5 us however little it does; six solves at n = 2592 with their reports 4209
+// us, 4000 so and with the second pass left out below).
+constexpr int FC_COLS = 512;  // PG_WIDE_N / 8
+template <class Val>
+struct ColFormed {
+    float2 *sv;  // FC_COLS, shared
+    Val val;
+    int64_t first, last;
+    __device__ __forceinline__ void stage(int64_t j0, int64_t j1)
+    {
+        if (j0 == first && j1 == last) return;
+        first = j0;
+        last = j1;
+        for (int64_t j = j0 + threadIdx.x; j < j1; j += PG_THREADS) sv[j - j0] = df_split(val(j));
+        __syncthreads();
+    }
+    __device__ __forceinline__ float2 at(int64_t j) const { return sv[j - first]; }
+};
+
+template <class Val>
+__device__ __forceinline__ void mv32_formed(const PgArgs &a, double *sm, float2 *sv, Val val)
+{
+    mv32_tiles(a, sm, ColFormed<Val>{sv, val, -1, -1});
 }
 
 __device__ __forceinline__ double warp_sum_d(double v)
@@ -456,8 +497,8 @@ __device__ void sum_dots(const PgArgs &a, int region, int j, double *h)
     __syncthreads();
 }
 
-// The residual r_e = res(e, b_e) of the CTA's own chunk into a.w and, as
-// float pairs, a.vf (the next preconditioner product's input); the chunk's
+// The residual r_e = res(e, b_e) of the CTA's own chunk as float pairs into a.vf
+// (the next preconditioner product's input); the chunk's
 // ||r||_inf (infinite if any r_e is not finite) and ||b||_inf into dp1[0],
 // dp1[1] by its owner.
 template <class Res>
@@ -468,7 +509,6 @@ __device__ __forceinline__ void store_residual(const PgArgs &a, int64_t e0, int6
     for (int64_t e = e0 + threadIdx.x; e < e1; e += PG_THREADS) {
         const double be = __ldg(a.b + e);
         const double re = res(e, be);
-        a.w[e] = re;
         a.vf[e] = df_split(re);
         rmax = fmax(rmax, fabs(re));
         bmax = fmax(bmax, fabs(be));
@@ -503,6 +543,9 @@ __global__ void __launch_bounds__(PG_THREADS, MINB) k_gmres_ir(PgArgs a)
     // the exact residual's group tree take all 1024
     __shared__ __align__(16) double smv[2 * MV_GROUPS * MV64_ROWS];
     __shared__ int s_ok;
+    // a lone small system: the preconditioner's products form their own vectors
+    constexpr bool FORM = MINB == 1;
+    __shared__ float2 sv[FORM ? FC_COLS : 1];
     int32_t tgt = 0;  // grid barrier target (thread 0)
     static_assert(MV_GROUPS * MV32_ROWS <= 2 * MV_GROUPS * MV64_ROWS, "shared product tile");
     constexpr int LDH = PG_MAXM + 1;
@@ -522,9 +565,14 @@ __global__ void __launch_bounds__(PG_THREADS, MINB) k_gmres_ir(PgArgs a)
     // x = M b (cold start); the exact residual's anchor needs ||A||_inf and
     // ||x||_inf up front, and the row sums of |A| share the product's phase
     if (a.cold) {
-        for (int64_t e = e0 + threadIdx.x; e < e1; e += PG_THREADS) a.vf[e] = df_split(__ldg(a.b + e));
-        if (!grid_sync(a, &s_ok, tgt)) return;
-        mv32_partial(a, smv);
+        if constexpr (FORM) {
+            mv32_formed(a, smv, sv, [&](int64_t j) { return __ldg(a.b + j); });
+        } else {
+            for (int64_t e = e0 + threadIdx.x; e < e1; e += PG_THREADS)
+                a.vf[e] = df_split(__ldg(a.b + e));
+            if (!grid_sync(a, &s_ok, tgt)) return;
+            mv32_partial(a, smv);
+        }
     }
     if (a.dd) mv64_partial<true>(a, nullptr, 1.0, smv);
     if (a.cold || a.dd) {
@@ -533,6 +581,7 @@ __global__ void __launch_bounds__(PG_THREADS, MINB) k_gmres_ir(PgArgs a)
         for (int64_t e = e0 + threadIdx.x; e < e1; e += PG_THREADS) {
             const double xe = a.cold ? sum_parts32(a, e) : __ldcg(a.x + e);
             if (a.cold) a.x[e] = xe;
+            if (a.Adf) a.Vf[e] = df_split(xe);
             if (a.dd) amax = fmax(amax, sum_parts(a, a.s64, e));
             xmax = fmax(xmax, fabs(xe));
         }
@@ -563,17 +612,15 @@ __global__ void __launch_bounds__(PG_THREADS, MINB) k_gmres_ir(PgArgs a)
         bool cheap = false;
         const double red = PG_CHEAP_RED < 0.0 ? 10.0 * a.tol_in : PG_CHEAP_RED;
         if (a.dd && eta_prev * red >= PG_CHEAP_ETA) {
-            if (a.Adf) {
-                for (int64_t e = e0 + threadIdx.x; e < e1; e += PG_THREADS)
-                    a.Vf[e] = df_split(__ldcg(a.x + e));
-                if (!grid_sync(a, &s_ok, tgt)) return;
+            if (a.Adf)  // a.Vf holds x
                 mv64df_partial(a, 1.0, smv);
-            } else {
+            else
                 mv64_partial<false>(a, a.x, 1.0, smv);
-            }
             if (!grid_sync(a, &s_ok, tgt)) return;
-            store_residual(a, e0, e1, owner, dp1, sred,
-                           [&](int64_t e, double be) { return be - sum_parts(a, a.s64, e); });
+            auto res = [&](int64_t e, double be) { return be - sum_parts(a, a.s64, e); };
+            if constexpr (FORM)
+                mv32_formed(a, smv, sv, [&](int64_t j) { return res(j, __ldg(a.b + j)); });
+            store_residual(a, e0, e1, owner, dp1, sred, res);
             if (!grid_sync(a, &s_ok, tgt)) return;
             const double rn = chunk_total(a, 1, 0, true, sred);
             const double bn = chunk_total(a, 1, 1, true, sred);
@@ -592,9 +639,12 @@ __global__ void __launch_bounds__(PG_THREADS, MINB) k_gmres_ir(PgArgs a)
             else
                 mv64_partial<false>(a, a.x, 1.0, smv);
             if (!grid_sync(a, &s_ok, tgt)) return;
-            store_residual(a, e0, e1, owner, dp1, sred, [&](int64_t e, double be) {
+            auto res = [&](int64_t e, double be) {
                 return a.dd ? residual_fx_at(a, be, e, fxc) : be - sum_parts(a, a.s64, e);
-            });
+            };
+            if constexpr (FORM)
+                mv32_formed(a, smv, sv, [&](int64_t j) { return res(j, __ldg(a.b + j)); });
+            store_residual(a, e0, e1, owner, dp1, sred, res);
             if (!grid_sync(a, &s_ok, tgt)) return;
             if (a.dd) {
                 const double rn = chunk_total(a, 1, 0, true, sred);
@@ -627,8 +677,10 @@ __global__ void __launch_bounds__(PG_THREADS, MINB) k_gmres_ir(PgArgs a)
             }
         }
         // V_0 = M r (raw), beta = ||V_0||
-        mv32_partial(a, smv);
-        if (!grid_sync(a, &s_ok, tgt)) return;
+        if constexpr (!FORM) {
+            mv32_partial(a, smv);
+            if (!grid_sync(a, &s_ok, tgt)) return;
+        }
         {
             double s = 0.0;
             for (int64_t e = e0 + threadIdx.x; e < e1; e += PG_THREADS) {
@@ -648,7 +700,7 @@ __global__ void __launch_bounds__(PG_THREADS, MINB) k_gmres_ir(PgArgs a)
         }
         for (int i = threadIdx.x; i <= m; i += PG_THREADS) sg[i] = i == 0 ? beta : 0.0;
         __syncthreads();
-        double sv = beta > 0.0 ? 1.0 / beta : 0.0;  // scale of the raw V_j
+        double vs = beta > 0.0 ? 1.0 / beta : 0.0;  // scale of the raw V_j
         int k = 0;
         bool bad = false;
         for (int j = 0; j < m; ++j) {
@@ -656,19 +708,21 @@ __global__ void __launch_bounds__(PG_THREADS, MINB) k_gmres_ir(PgArgs a)
             double *u = a.V + (int64_t)(j + 1) * a.ldv;
             // w = A v_j (the FP64 matrix, or its float-pair copy and a.Vf)
             if (a.Adf)
-                mv64df_partial(a, sv, smv);
+                mv64df_partial(a, vs, smv);
             else
-                mv64_partial<false>(a, Vj, sv, smv);
+                mv64_partial<false>(a, Vj, vs, smv);
             if (!grid_sync(a, &s_ok, tgt)) return;
             for (int64_t e = e0 + threadIdx.x; e < e1; e += PG_THREADS) {
-                Vj[e] = __ldcg(Vj + e) * sv;  // v_j normalised in place (own chunk)
-                const double we = sum_parts(a, a.s64, e);
-                a.w[e] = we;
-                a.vf[e] = df_split(we);
+                Vj[e] = __ldcg(Vj + e) * vs;  // v_j normalised in place (own chunk)
+                if (!FORM) a.vf[e] = df_split(sum_parts(a, a.s64, e));
             }
-            if (!grid_sync(a, &s_ok, tgt)) return;
             // u = M w, then two classical Gram-Schmidt passes and the norm
-            mv32_partial(a, smv);
+            if constexpr (FORM) {
+                mv32_formed(a, smv, sv, [&](int64_t j) { return sum_parts(a, a.s64, j); });
+            } else {
+                if (!grid_sync(a, &s_ok, tgt)) return;
+                mv32_partial(a, smv);
+            }
             if (!grid_sync(a, &s_ok, tgt)) return;
             for (int64_t e = e0 + threadIdx.x; e < e1; e += PG_THREADS) u[e] = sum_parts32(a, e);
             __syncthreads();
@@ -681,10 +735,10 @@ __global__ void __launch_bounds__(PG_THREADS, MINB) k_gmres_ir(PgArgs a)
                 u[e] = s;
             }
             __syncthreads();
-            if (owner) chunk_dots(a, 1, j, u, e0, e1);
+            if (owner) chunk_dots(a, 1, j + 1, u, e0, e1);  // and u . u
             if (!grid_sync(a, &s_ok, tgt)) return;
-            sum_dots(a, 1, j, sh2);
-            {
+            sum_dots(a, 1, j + 1, sh2);
+            auto second_pass = [&]() {
                 double s2 = 0.0;
                 for (int64_t e = e0 + threadIdx.x; e < e1; e += PG_THREADS) {
                     double s = __ldcg(u + e);
@@ -694,11 +748,25 @@ __global__ void __launch_bounds__(PG_THREADS, MINB) k_gmres_ir(PgArgs a)
                     if (a.Adf) a.Vf[e] = df_split(s);
                     s2 = fma(s, s, s2);
                 }
-                s2 = block_sum_all(s2, sred);
+                return s2;
+            };
+            // ||u||^2 after the second pass is u . u - |h2|^2, to rounding as long as
+            // that pass takes little away; then the pass itself, and a barrier, are
+            // only needed if another iteration follows
+            double h2 = 0.0;
+            for (int i = threadIdx.x & 31; i <= j; i += 32) h2 = fma(sh2[i], sh2[i], h2);
+            h2 = warp_sum_d(h2);
+            const double uu = sh2[j + 1];
+            const bool direct = h2 <= 1e-3 * uu;  // (false if not a number)
+            double hn;
+            if (direct) {
+                hn = sqrt(uu - h2);
+            } else {
+                const double s2 = block_sum_all(second_pass(), sred);
                 if (owner && threadIdx.x == 0) dp2[nslot] = s2;
+                if (!grid_sync(a, &s_ok, tgt)) return;
+                hn = sqrt(chunk_total(a, 2, nslot, false, sred));
             }
-            if (!grid_sync(a, &s_ok, tgt)) return;
-            const double hn = sqrt(chunk_total(a, 2, nslot, false, sred));
             // column j of H, previous rotations, the new rotation (every CTA, same order)
             double res = 0.0;
             if (threadIdx.x == 0) {
@@ -730,8 +798,12 @@ __global__ void __launch_bounds__(PG_THREADS, MINB) k_gmres_ir(PgArgs a)
                 bad = true;
                 break;
             }
-            sv = hn > 0.0 ? 1.0 / hn : 0.0;
+            vs = hn > 0.0 ? 1.0 / hn : 0.0;
             if (res <= a.tol_in * beta || hn == 0.0) break;
+            if (direct && j + 1 < m) {  // u is wanted after all
+                second_pass();
+                if (!grid_sync(a, &s_ok, tgt)) return;
+            }
         }
         if (bad) {
             if (blockIdx.x == 0 && threadIdx.x == 0) atomicOr(a.status, ST_NONFINITE);
@@ -753,6 +825,7 @@ __global__ void __launch_bounds__(PG_THREADS, MINB) k_gmres_ir(PgArgs a)
                 for (int i = 0; i < k; ++i) s = fma(sy[i], __ldcg(a.V + (int64_t)i * a.ldv + e), s);
                 const double xe = __ldcg(a.x + e) + s;
                 a.x[e] = xe;
+                if (a.Adf) a.Vf[e] = df_split(xe);
                 dmax = fmax(dmax, fabs(s));
                 xmax = fmax(xmax, fabs(xe));
                 if (!isfinite(s) || !isfinite(xe)) dmax = INFINITY;
@@ -806,6 +879,7 @@ bool pg_supported(const Ctx &c) { return c.factored_prec != NRS_FP64 && c.max_in
 
 // systems from this order up stream their matrices from HBM in the products
 static constexpr int64_t PG_WIDE_N = 4096;
+static_assert(PG_WIDE_N <= 8 * FC_COLS, "a split's columns fit");
 
 static const void *pg_kernel(const Ctx &c)
 {
@@ -835,27 +909,25 @@ int pg_max_coresident(const Ctx &c)
 
 size_t pg_dpart_doubles(int max_inner) { return (size_t)3 * PG_MAXCH * (max_inner + 2); }
 
-// The number of column splits of a product of n columns with rc row tiles on
-// a grid of G CTAs: from lo on, and from as many as fit one wave, the smallest
-// whose rc s tiles fill their last wave to 97 %, else the best fill.  Every
-// element of the product is the sum of s partial sums, read one after the
-// other, so a split keeps at least PG_MIN_COLS columns (n = 288 on 152 CTAs
-// had taken 60 splits: 187 us a solve; 142 with 9 and two barriers fewer).
+// The number of column splits of a product of n columns with rc row tiles on a
+// grid of G CTAs, from lo on: the one of least cost, waves of tiles times their
+// columns at t clocks each, plus the sum of the splits' partial results, which
+// every element's reader loads one after the other (eight in flight: 175 clocks
+// a split).  A split keeps at least PG_MIN_COLS columns.  (With splits until the
+// last wave was full to 97 %, whatever their number, n = 288 on 152 CTAs took 60:
+// 187 us a solve; 142 with 9 and two barriers fewer.)
 constexpr int PG_MIN_COLS = 32;
-static int pick_splits(int64_t n, int64_t rc, int G, int lo)
+static int pick_splits(int64_t n, int64_t rc, int G, int lo, int64_t t)
 {
     const int hi = (int)std::max<int64_t>(lo, std::min<int64_t>(64, n / PG_MIN_COLS));
-    lo = std::max(lo, std::min(hi, (int)(G / rc)));
     int best = lo;
-    double best_fill = -1.0;
+    int64_t least = INT64_MAX;
     for (int s = lo; s <= hi; ++s) {
-        const int64_t t = rc * s;
-        const double fill = (double)t / (double)(ceil_div(t, G) * G);
-        if (fill > best_fill + 1e-12) {
-            best_fill = fill;
+        const int64_t cost = ceil_div(rc * s, G) * ceil_div(n, s) * t + 175 * s;
+        if (cost < least) {
+            least = cost;
             best = s;
         }
-        if (fill >= 0.97) break;
     }
     return best;
 }
@@ -874,7 +946,6 @@ cudaError_t launch_gmres_persistent(Ctx &c, const double *b, double *x, bool col
     a.b = b;
     a.x = x;
     a.V = c.d_V;
-    a.w = c.d_w;
     a.part = c.d_part;
     a.part32 = c.d_part32;
     a.part_fx = c.d_part_fx;
@@ -894,16 +965,18 @@ cudaError_t launch_gmres_persistent(Ctx &c, const double *b, double *x, bool col
     a.cold = cold ? 1 : 0;
     a.rc64 = (int)ceil_div(c.n, MV64_ROWS);
     a.rc32 = (int)ceil_div(c.n, MV32_ROWS);
-    // column splits (at n = 27648: 432 row tiles on 304 CTAs fill 71 % of the
-    // last wave with one split, 99.5 % with seven); at least 8 for the FP32
-    // product: each partial sum then covers at most n / 8 columns before the
-    // splits are added in FP64
-    a.s64 = pick_splits(c.n, a.rc64, G, 1);
-    a.s32 = pick_splits(c.n, a.rc32, G, 8);
+    // column splits; at least 8 for the FP32 product: each partial sum then covers
+    // at most n / 8 columns before the splits are added in FP64.  A tile's column
+    // of 512 bytes takes 70 clocks with three CTAs an SM streaming from HBM; from
+    // L2 the FP64 pipe takes 32 for it, the FP32 product 13
+    const bool lone = pg_kernel(c) == (const void *)k_gmres_ir<1>;
+    a.s64 = pick_splits(c.n, a.rc64, G, 1, lone ? 32 : 70);
+    a.s32 = pick_splits(c.n, a.rc32, G, 8, lone ? 13 : 70);
     a.s64 = (int)std::min<int64_t>(a.s64, c.n);
     a.s32 = (int)std::min<int64_t>(a.s32, c.n);
     a.cps64 = ceil_div(c.n, a.s64);
     a.cps32 = ceil_div(c.n, a.s32);
+    if (lone && a.cps32 > FC_COLS) return cudaErrorInvalidValue;  // (n < 8 FC_COLS there)
     // chunk owners: at most PG_MAXCH CTAs, about 64 elements each
     a.dch = (int)std::max<int64_t>(1, std::min<int64_t>(std::min<int64_t>(PG_MAXCH, G),
                                                         ceil_div(c.n, 64)));

@@ -30,15 +30,24 @@ using namespace tcp;
 // PRESPLIT: the panels arrive already split (hi in tmA/tmB, lo in tmAl/tmBl,
 // as the prep stores them for this kernel), so the tiles go to the tensor
 // cores as loaded; otherwise the FP32 panels are split here.
-template <bool PRESPLIT>
-__global__ void __launch_bounds__(128, 1)
+// TILED: a tile of M goes through shared memory by TMA, once the products have
+// read the operands there; otherwise every thread reads, subtracts and writes 16
+// columns of its row at a time, the next 16 on their way.  The plain loads in
+// flight are limited by what shared memory leaves to the L1 cache (four times as
+// many, or twice the warps, made a step of n = 5115 no faster or slower), the
+// copies are not: with more than a wave of tiles, or several chains at once, the
+// copies win (n = 5115: 61 to 46 us a step; a batch of node problems 24.1 to 23.2
+// ms); with a lone wave the tile's own latency counts, and they lose (n = 2406:
+// 17 against 20 us).
+template <bool PRESPLIT, bool TILED>
+__global__ void __launch_bounds__(128, TILED ? 4 : 1)
     k_tc_gj_update(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                    const __grid_constant__ CUtensorMap tmAl, const __grid_constant__ CUtensorMap tmBl,
-                   int64_t n, float *__restrict__ M, int64_t lda, int32_t *status, int64_t skip0,
+                   const __grid_constant__ CUtensorMap tmM, int64_t n, float *__restrict__ M, int64_t lda, int32_t *status, int64_t skip0,
                    int64_t kblk)
 {
     extern __shared__ uint8_t smem_raw[];
-    __shared__ uint64_t bar_load[2], bar_mma[2];
+    __shared__ uint64_t bar_load[2], bar_mma[2], bar_tile;
     __shared__ uint32_t tmem_slot;
     __shared__ int s_ok;
     uint8_t *base = reinterpret_cast<uint8_t *>(
@@ -50,8 +59,17 @@ __global__ void __launch_bounds__(128, 1)
     float *sBl = reinterpret_cast<float *>(base + 3 * TC_TILE_BYTES);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t row0 = (int64_t)blockIdx.x * TC_BM, col0 = (int64_t)blockIdx.y * TC_BN;
+    // the whole tile of M can go through shared memory: it meets neither the block
+    // row and column kblk nor the block at skip0, which others may write meanwhile,
+    // and the store, which is cut off at n in units of 16 bytes, leaves the padding
+    // rows below n alone
+    auto meets = [](int64_t t0, int64_t b0) { return t0 < b0 + 64 && b0 < t0 + TC_BM; };
+    const bool whole = TILED && (row0 + TC_BM <= n || (n & 3) == 0) && !meets(row0, kblk) && !meets(col0, kblk) &&
+                       !(meets(row0, skip0) && meets(col0, skip0));
 
     if (threadIdx.x == 0) {
+        if (whole) tma_prefetch_2d(&tmM, (int)row0, (int)col0);
+        mbar_init(&bar_tile, 1);
         for (int i = 0; i < 2; ++i) {
             mbar_init(&bar_load[i], 1);
             mbar_init(&bar_mma[i], 1);
@@ -129,11 +147,12 @@ __global__ void __launch_bounds__(128, 1)
         }
     }
     __syncthreads();
-    bool ok = s_ok != 0;
-    if (ok && !mbar_wait(&bar_mma[1], 0)) {
+    if (s_ok && !mbar_wait(&bar_mma[1], 0)) {
         atomicOr(status, ST_TIMEOUT);
-        ok = false;
+        s_ok = 0;
     }
+    __syncthreads();
+    const bool ok = s_ok != 0;  // the same for every thread
     if (!ok && threadIdx.x == 0) {
         // bounded waits for whatever copies or MMAs may still be in flight
         mbar_wait(&bar_load[0], 0);
@@ -142,7 +161,38 @@ __global__ void __launch_bounds__(128, 1)
         mbar_wait(&bar_mma[1], 0);
     }
     tc_fence_after();
-    if (ok) {
+    if (ok && whole) {
+        // the products have read the operands: their 64 KB take the tile of M
+        float *tile = sA;
+        if (threadIdx.x == 0) {
+            mbar_expect_tx(&bar_tile, TC_BM * TC_BN * 4);
+            tma_load_2d(tile, &tmM, (int)row0, (int)col0, &bar_tile);
+        }
+        if (__all_sync(0xffffffffu, mbar_wait(&bar_tile, 0))) {
+            float *p = tile + warp * 32 + lane;
+#pragma unroll 1
+            for (int c = 0; c < TC_BN; c += 16) {
+                uint32_t v[16];
+                tmem_ld_16cols(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c, v);
+#pragma unroll
+                for (int j = 0; j < 16; ++j) p[(c + j) * TC_BM] -= __uint_as_float(v[j]);
+            }
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        } else {
+            atomicOr(status, ST_TIMEOUT);
+            s_ok = 0;
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            if (s_ok) {
+                tma_store_2d(&tmM, tile, (int)row0, (int)col0);
+                bulk_commit();
+                bulk_wait_all();
+            } else {
+                mbar_wait(&bar_tile, 0);  // (bounded) for the copy in flight
+            }
+        }
+    } else if (ok) {
         const int64_t row = row0 + warp * 32 + lane;
         // the 64 x 64 block at (skip0, skip0) is updated separately (lookahead)
         const bool row_skip = row >= skip0 && row < skip0 + 64;
@@ -261,32 +311,31 @@ bool launch_tc_rank64(Ctx &c, float *M, int64_t lda, int64_t n, const float *Cb,
 {
     if (prec != NRS_TF32) return false;
     const bool split = Cb_lo != nullptr;
-    CUtensorMap a, b, al, bl;
+    CUtensorMap a, b, al, bl, m;
     if (!make_panel_map(&a, Cb, n) || !make_panel_map(&b, Rt, n)) return false;
     if (split && (!make_panel_map(&al, Cb_lo, n) || !make_panel_map(&bl, Rt_lo, n))) return false;
     if (!split) {
         al = a;
         bl = b;
     }
+    dim3 grid((unsigned)ceil_div(n, TC_BM), (unsigned)ceil_div(n, TC_BN));
+    // three CTAs fit an SM (a matrix that no tensor map describes: plain loads)
+    const bool tiled = (c.pg_shared || (int64_t)grid.x * grid.y > 3 * (int64_t)c.num_sms) &&
+                       make_matrix_map(&m, M, n, lda);
+    if (!tiled) m = a;
+    auto kernel = split ? (tiled ? k_tc_gj_update<true, true> : k_tc_gj_update<true, false>)
+                        : (tiled ? k_tc_gj_update<false, true> : k_tc_gj_update<false, false>);
     static bool attr = false;
     if (!attr) {
-        cudaFuncSetAttribute(k_tc_gj_update<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             TC_SMEM);
-        cudaFuncSetAttribute(k_tc_gj_update<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             TC_SMEM);
-        cudaFuncSetAttribute(k_tc_gj_update<false>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                             cudaSharedmemCarveoutMaxShared);
-        cudaFuncSetAttribute(k_tc_gj_update<true>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                             cudaSharedmemCarveoutMaxShared);
+        for (auto k : {k_tc_gj_update<true, true>, k_tc_gj_update<true, false>,
+                       k_tc_gj_update<false, true>, k_tc_gj_update<false, false>}) {
+            cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM);
+            cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                 cudaSharedmemCarveoutMaxShared);
+        }
         attr = true;
     }
-    dim3 grid((unsigned)ceil_div(n, TC_BM), (unsigned)ceil_div(n, TC_BN));
-    if (split)
-        k_tc_gj_update<true><<<grid, 128, TC_SMEM, c.stream>>>(a, b, al, bl, n, M, lda, c.d_status,
-                                                                skip0, kblk);
-    else
-        k_tc_gj_update<false><<<grid, 128, TC_SMEM, c.stream>>>(a, b, al, bl, n, M, lda, c.d_status,
-                                                                 skip0, kblk);
+    kernel<<<grid, 128, TC_SMEM, c.stream>>>(a, b, al, bl, m, n, M, lda, c.d_status, skip0, kblk);
     c.launches += 1;
     return true;
 }

@@ -35,6 +35,9 @@ constexpr int AS_CHUNK = 512;
 // up to three of its CTAs still fit beside one (the order of the sums over q
 // does not depend on the chunk)
 constexpr int AS64_CHUNK = 128;
+// order from which the FP64 assembly beside a lone factorisation takes the
+// integer form
+constexpr int64_t ASM_INT_MIN_N = 4096;
 
 struct Acc6 {
     double xx, xy, xz, yy, yz, zz;
@@ -564,14 +567,15 @@ void launch_assemble(Ctx &c, const D4 *x_lab, double *A64, float *A32, int64_t l
     if (side) {
         // beside the factorisation: a few CTAs of four warps per SM, claiming
         // tiles, so that the factorisation's kernels (one CTA per SM each) still
-        // find room on every SM.  A lone one-level factorisation outlasts the
-        // assembly either way, and its chain of latency-bound kernels suffers
+        // find room on every SM.  A lone small one-level factorisation outlasts
+        // the assembly either way, and its chain of latency-bound kernels suffers
         // more from the integer form's issue slots and registers than from the
         // FP64 form's longer run (single swimmer's step: 3.18 ms with the FP64
         // form, 3.27 with the integer one); among the chains of a batch (32
-        // reduced nodes: 37.1 and 25.2 ms) and beside the two-level updates the
-        // integer form is the better one.
-        if (!c.pg_shared && c.n < GJ2_MIN_N) kernel = k_assemble64<false>;
+        // reduced nodes: 37.1 and 25.2 ms), beside the two-level updates and beside
+        // one-level updates that take longer than the chain (n = 5115: the
+        // assembly alone 2.6 and 1.2 ms) the integer form is the better one.
+        if (!c.pg_shared && c.n < ASM_INT_MIN_N) kernel = k_assemble64<false>;
         grid = std::min<int64_t>(tiles, (int64_t)c.asm_side_ctas * c.num_sms);
     }
     kernel<<<(unsigned)grid, AS_THREADS, 0, s>>>(

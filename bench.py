@@ -87,8 +87,11 @@ TF32_OVER_BF16 = 1.1 / 2.25      # nominal dense TF32 / BF16 tensor throughput
 SM_COUNT_NOMINAL = 152
 FP32_LANES_PER_SM = 128
 PAIR_INSTR = 20                  # FP32-pipe instructions per (force, quadrature) pair
-ASM64_OPS_PER_PAIR = 40          # FP64 operations per pair of the bit-exact assembly
-RES_OPS_PER_ENTRY = 3           # FP64 operations per matrix entry of the extended residual
+# Work counted in FP64 operations, most of which the kernels do on the integer
+# pipe (correctly rounded, or exactly): a fraction of the FP64 pipe's rate above 1
+# means that much more than that pipe alone could do
+ASM64_OPS_PER_PAIR = 40          # per pair of the bit-exact assembly
+RES_OPS_PER_ENTRY = 3            # per matrix entry of the extended residual
 TOL = 1e-10
 
 
@@ -352,8 +355,8 @@ def rooflines(ph_ms, ph_spans, n, pairs, peaks, peak_src, sm_mhz, solve_stats, p
                   products, exact from A in FP64 or in working precision from its
                   float-pair copy, and the GMRES products: 8 bytes an entry each)
                   + (outer + inner + 1) 4 n^2 bytes of M; + 8 n^2 (||A||_inf, once
-                  per launch); exact x 3 n^2 (extended residual: product, its error,
-                  the error sum; the products' sum on the integer pipe) + n^2
+                  per launch); exact x 3 n^2 (extended residual: product, its error
+                  and the error sum, all on the integer pipe) + n^2
                   (||A||_inf) + (inner + working) x n^2 (the GMRES and residual
                   products, when in FP64) FP64 operations.  Without the residual
                   counts, every refinement step counts one exact residual."""
@@ -443,7 +446,8 @@ def rooflines(ph_ms, ph_spans, n, pairs, peaks, peak_src, sm_mhz, solve_stats, p
             "peak_source": "derived: nominal FP64 1.25 TFLOP/s = 625 G FP64 ops/s at 2070 MHz, "
                            "scaled to the sampled clock",
             "work_per_launch": ops, "work_unit": "FP64 operations (40 per pair; square root and "
-                                                 "division counted once each)",
+                                                 "division counted once each; the products, "
+                                                 "roots and reciprocals on the integer pipe)",
             "pairs_per_s": p64 / t, "pairs_evaluated_per_launch": p64,
             "pairs_kept_per_launch": pairs - p64, "ms_per_launch": t * 1e3,
             "launches": ph_spans["assemble"], "traffic": _traffic("k_assemble64", n)}
@@ -812,7 +816,8 @@ def tracers_line(nrs, args, timer, count=2000, steps=3, warm=1):
             "s_per_step": float(np.mean(ms)) / 1e3, "steps": steps,
             "velocity_ms": t * 1e3, "velocity_pairs_per_s": pairs / t,
             "velocity_fp64_gops": pairs * 52 / t / 1e9,
-            "velocity_note": "52 FP64 operations per (tracer, quadrature point) pair; two "
+            "velocity_note": "work counted as 52 FP64 operations per (tracer, quadrature point) "
+                             "pair, done in 19 fused multiply-adds and integer steps; two "
                              "evaluations per step",
             "max_tracer_displacement": moved}
 

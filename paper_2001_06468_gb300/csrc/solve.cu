@@ -92,7 +92,7 @@ __device__ __forceinline__ bool wait_flag(const int32_t *flags, int64_t j, int32
 // tid mod 64, 16 columns), and the diagonal block is solved with the inverses
 // of its 32 x 32 triangles (lu.cu), three 32 x 32 products by eight lanes a
 // row, instead of 64 dependent steps with a division each (446 and 1197 us a
-// solve for n = 2406 so).
+// solve for n = 2406; 165 each so).
 constexpr int TR_THREADS = 256, TR_HB = 32;
 
 // sum over the eight lanes of a row (fixed order, every lane gets it)
@@ -695,6 +695,8 @@ static void norms(Ctx &c, const double *x, const double *b)
     c.launches += 2;
 }
 
+constexpr int64_t FX_HBM_N = 4096;  // 8 n^2 bytes are more than L2 holds from here
+
 // r = b - A x with the FP64 matrix: to about u^2 (exact products, fx_madd)
 // unless the context asks for a plain FP64 residual.  The exact one leaves
 // ||A||_inf, ||x||_inf (its anchor), ||b||_inf and ||r||_inf in scal.
@@ -704,14 +706,21 @@ static void residual(Ctx &c, const double *x, const double *b, double *r)
         gemv(c, x, b, r);
         return;
     }
-    const int64_t cps = ceil_div(c.n, c.splits64);
-    dim3 grid((unsigned)ceil_div(c.n, 2 * MV_THREADS), (unsigned)c.splits64);
+    // two blocks an SM, as the plain products; six where the matrix comes from HBM
+    // (n = 5115: 229 us with two, 113 with six, the mixed solve 6408 and 6302 us;
+    // n = 2592, from L2: six solves with reports 4004 and 4051 us, the sums of
+    // more splits taking longer).  The sums are exact however they are split.
+    const int64_t rowblocks = ceil_div(c.n, 2 * MV_THREADS);
+    const int64_t blocks = (c.n < FX_HBM_N ? 2 : 6) * (int64_t)c.num_sms;
+    const int splits = (int)std::min<int64_t>(std::min<int64_t>(64, c.n), ceil_div(blocks, rowblocks));
+    const int64_t cps = ceil_div(c.n, splits);
+    dim3 grid((unsigned)rowblocks, (unsigned)splits);
     c.tbeg(PH_GEMV);
     norms(c, x, b);
     k_gemv_part_fx<<<grid, MV_THREADS, 0, c.stream>>>(c.n, c.d_A64, c.lda, x, c.d_scal, c.d_part_fx,
                                                       c.d_part, cps);
     k_gemv_finish_fx<<<(unsigned)ceil_div(c.n, 32), 32 * FXF_WARPS, 0, c.stream>>>(
-        c.n, c.d_part_fx, c.d_part, c.splits64, c.d_scal, b, r, c.d_scal + SC_RN);
+        c.n, c.d_part_fx, c.d_part, splits, c.d_scal, b, r, c.d_scal + SC_RN);
     c.tend(PH_GEMV);
     c.launches += 2;
 }

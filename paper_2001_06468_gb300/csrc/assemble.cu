@@ -22,8 +22,8 @@
 
 #include <algorithm>
 
-#include "fp64_int.cuh"
 #include "nrs_internal.cuh"
+#include "stokeslet_int.cuh"
 
 namespace nrs {
 
@@ -39,45 +39,9 @@ constexpr int AS64_CHUNK = 128;
 // integer form
 constexpr int64_t ASM_INT_MIN_N = 4096;
 
-struct Acc6 {
-    double xx, xy, xz, yy, yz, zz;
-};
-
-// FP64 additions and products as fused multiply-adds: GB300 issues an FP64
-// fused multiply-add every 64 clocks per scheduler, a plain add or multiply
-// every 76.  `one` is 1.0 and `nz` is -0.0, passed at run time so that the
-// compiler does not turn them back; a 1 + b and a b + (-0.0) round exactly as
-// a + b and a b do (signed zeros included).
-struct FmaOps {
-    double one, nz;
-    __device__ __forceinline__ double add(double a, double b) const { return __fma_rn(a, one, b); }
-    __device__ __forceinline__ double sub(double a, double b) const { return __fma_rn(b, -one, a); }
-    __device__ __forceinline__ double mul(double a, double b) const { return __fma_rn(a, b, nz); }
-};
-
-// A quadrature point staged for the pair loop: its weight also as a
-// significand for the integer products (shifted left by one, sign and
-// exponent field), usable when `ok`.
-struct alignas(16) StagedX {
-    double x, y, z, w;
-    uint64_t w2;
-    uint32_t wf, ok;
-};
-
 __device__ __forceinline__ StagedX stage_point(const D4 &p)
 {
-    StagedX v;
-    v.x = p.x;
-    v.y = p.y;
-    v.z = p.z;
-    v.w = p.w;
-    const Sig sw = unpack(p.w);
-    v.w2 = sw.m << 1;
-    v.wf = sw.f;
-    // 2^-200 <= |w| < 2^200 (zero, subnormal and non-finite weights excluded)
-    const uint32_t ex = (sw.f >> 20) & 0x7ffu;
-    v.ok = ex - 823u < 400u;
-    return v;
+    return stage_weighted(p.x, p.y, p.z, p.w);
 }
 
 __device__ __forceinline__ float2 df_split_int(double v)
@@ -142,56 +106,6 @@ __device__ __forceinline__ Acc6 terms_fp64(double mx, double my, double mz, cons
     v.yy = __dmul_rn(__dmul_rn(__dadd_rn(__dmul_rn(ry, ry), dg), s), w);
     v.yz = __dmul_rn(__dmul_rn(__dmul_rn(ry, rz), s), w);
     v.zz = __dmul_rn(__dmul_rn(__dadd_rn(__dmul_rn(rz, rz), dg), s), w);
-    return v;
-}
-
-// Squared distances below this component count as zero in terms_int.
-constexpr uint32_t kTinyHi = 873u << 20;  // 2^-150
-
-__device__ __forceinline__ bool tiny(double r)
-{
-    return (hi32(double_bits(r)) & 0x7fffffffu) < kTinyHi;
-}
-
-// The terms of one pair, without a branch.  The FP64 pipe bounds this kernel,
-// so it is left the 16 additions and subtractions; the square root, the
-// reciprocal and the 18 products r_j r_k, s and w run beside it on the integer
-// pipe, rounded identically (fp64_int.cuh).  A component of r below 2^-150 is
-// taken as zero (then a product with it is a zero, whose sign does not matter:
-// a sum starts at +0).  odd = 1: some component was; 2 and more: the general
-// path is needed.
-__device__ __forceinline__ Acc6 terms_int(double mx, double my, double mz, const StagedX &X,
-                                          double eps2, double two_e2, const FmaOps &op, int &odd)
-{
-    const double rx = op.sub(mx, X.x), ry = op.sub(my, X.y), rz = op.sub(mz, X.z);
-    const bool tx = tiny(rx), ty = tiny(ry), tz = tiny(rz);
-    const Sig ux = unpack(rx), uy = unpack(ry), uz = unpack(rz);
-    bool bad = !X.ok;
-    const Sig pxx = mul_sig(ux, ux.m << 1, ux.f, bad);
-    const Sig pyy = mul_sig(uy, uy.m << 1, uy.f, bad);
-    const Sig pzz = mul_sig(uz, uz.m << 1, uz.f, bad);
-    const double xx = tx ? 0.0 : pack(pxx), yy = ty ? 0.0 : pack(pyy), zz = tz ? 0.0 : pack(pzz);
-    const double r2 = op.add(op.add(xx, yy), zz);
-    const double rho = op.add(r2, eps2);
-    const double dg = op.add(r2, two_e2);
-    // rho in [2^-100, 2^100)
-    bad |= (hi32(double_bits(rho)) - (923u << 20)) >= (200u << 20);
-    const Sig s = inv_rho_sqrt(rho, bad);
-    const uint64_t s2 = s.m << 1;
-    auto term = [&](const Sig &p) {
-        return pack(mul_sig(mul_sig(p, s2, s.f, bad), X.w2, X.wf, bad));
-    };
-    Acc6 v;
-    v.xx = term(unpack(op.add(xx, dg)));
-    v.yy = term(unpack(op.add(yy, dg)));
-    v.zz = term(unpack(op.add(zz, dg)));
-    const double xy = term(mul_sig(ux, uy.m << 1, uy.f, bad));
-    const double xz = term(mul_sig(ux, uz.m << 1, uz.f, bad));
-    const double yz = term(mul_sig(uy, uz.m << 1, uz.f, bad));
-    v.xy = tx || ty ? 0.0 : xy;
-    v.xz = tx || tz ? 0.0 : xz;
-    v.yz = ty || tz ? 0.0 : yz;
-    odd = (bad ? 2 : 0) | (tx || ty || tz ? 1 : 0);
     return v;
 }
 

@@ -119,7 +119,7 @@ NRS_HD double pack(const Sig &s)
 
 // a b rounded: a.m shifted left by 10 (63 bits), b given shifted left by 1, so
 // that the top 64 bits of the 128-bit product hold 52 or 53 bits of it and
-// every partial sum fits 64 bits.
+// every partial sum fits 64 bits.  At most one of the significands is 2^53.
 NRS_HD Sig mul_sig(const Sig &a, uint64_t b2, uint32_t bf, bool &tie)
 {
     const uint64_t A = a.m << 10;
@@ -229,7 +229,10 @@ NRS_HD Sig inv_rho_sqrt(double rho_d, bool &tie)
                             hi32(m2) * lo32(p.m);
         s += th >> 31;
     }
-    return Sig{s, (2045u << 20) - p.f};
+    // 2^53 (p a power of two) becomes 2^52 and one more in the exponent: a product
+    // with it may meet another factor of 2^53
+    const uint32_t carry = hi32(s) >> 21;
+    return Sig{s - ((uint64_t)carry << 52), (2045u << 20) - p.f + (carry << 20)};
 }
 
 // v = hi + lo as two floats: hi the nearest float (a tie away from zero), lo

@@ -87,3 +87,29 @@ def test_far_and_non_finite_pairs_take_the_general_path(terms, value, where):
             x[:, k] *= rng.uniform(1.1, 1.9, len(x)) * rng.choice([-1.0, 1.0], len(x))
     _, odd = terms(x, X, e2)
     assert np.all(odd >= 2)
+
+
+def test_a_carry_in_a_product_where_the_reciprocal_is_a_power_of_two(terms):
+    # r_j r_k = (1 - (i 2^-52)^2) 2^c rounds up to 2^c and rho is 4^k exactly: both
+    # factors of the next product have rounded up to a power of two
+    x, X, e2 = [], [], []
+    for k in range(-8, 9):
+        for c in range(0, 12):
+            for i in (1, 2, 3, 5, 100):
+                for axes in ((0, 1, 2), (1, 0, 2), (2, 0, 1), (0, 2, 1)):
+                    for r3 in (0.0, 2.0 ** (k - 6)):
+                        r = np.zeros(3)
+                        r[axes[0]] = (1.0 + i * 2.0 ** -52) * 2.0 ** (k - 1)
+                        r[axes[1]] = (1.0 - i * 2.0 ** -52) * 2.0 ** (k - 2 - c)
+                        r[axes[2]] = r3
+                        r2 = (r[0] * r[0] + r[1] * r[1]) + r[2] * r[2]
+                        if r2 + (4.0 ** k - r2) == 4.0 ** k:
+                            x.append(r)
+                            X.append([0.0, 0.0, 0.0, 0.7])
+                            e2.append(4.0 ** k - r2)
+    x, X, e2 = np.array(x), np.array(X), np.array(e2)
+    assert len(x) > 1000
+    got, odd = terms(x, X, e2)
+    want = _definition(x, X, e2)
+    assert np.all(odd < 2)  # (a zero component: 1)
+    assert np.array_equal(got, want)

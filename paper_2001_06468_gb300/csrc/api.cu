@@ -241,10 +241,10 @@ nrs_status do_factor(Ctx *c, int prec)
 nrs_status do_segments_and_assemble(Ctx *c, const D4 *x_lab, const D4 *Xw_lab, bool write_lo = true,
                                     bool from_state = false, bool wait64 = false)
 {
+    // (joins an earlier FP64 assembly, which must not overlap this one)
     nrs::launch_gather(*c, Xw_lab, c->d_seg_ptr, c->d_perm);
     float *a32 = (c->factor_prec == NRS_FP64 || !write_lo) ? nullptr : c->d_A32;
     if (a32 && c->factored_prec != NRS_FP64) c->factored_prec = -1;
-    nrs::join_assembly(*c);  // an earlier FP64 assembly must not overlap this one
     if (a32 && c->lo_eval == 0) {
         // the FP32 copy first, alone on the GPU, so the factorisation can start;
         // then the FP64 matrix on the side stream beside the factorisation,
@@ -395,6 +395,9 @@ namespace {
 nrs_status step_graph(Ctx *c, const nrs_shapes *s0, const nrs_shapes *sh, double dt, double *sol,
                       nrs_step_report *report)
 {
+    // an assembly still on the side stream: neither the capture nor the replay
+    // may meet it
+    nrs::join_assembly(*c);
     Ctx::GraphKey key{{s0->xi, s0->Xiw, s0->xidot, sh->xi, sh->Xiw, sh->xidot}, dt,
                       report != nullptr};
     if (!c->gexec || !(key == c->gkey)) {

@@ -83,6 +83,7 @@ __global__ void k_kinematics(int64_t N, int64_t Q, int64_t F, const D4 *__restri
 void launch_kinematics(Ctx &c, const D4 *xi, const D4 *Xiw, const D4 *xidot, D4 *x, D4 *Xw,
                        double *b)
 {
+    if (x == c.d_x) join_assembly(c);  // (the side stream reads it)
     int64_t total = c.N + c.Q + 6 * c.F;
     int threads = 256;
     c.tbeg(PH_KINEMATICS);
@@ -623,6 +624,7 @@ __global__ void k_sort_segments(int64_t N, const int32_t *__restrict__ seg_ptr,
 
 void launch_segments(Ctx &c, const int32_t *nn, int32_t *seg_ptr, int32_t *perm)
 {
+    join_assembly(c);  // an assembly still on the side stream reads seg_ptr
     int threads = 256;
     c.tbeg(PH_SEGMENTS);
     cudaMemsetAsync(c.d_cursor, 0, sizeof(int32_t) * (c.N + 1), c.stream);
@@ -668,6 +670,7 @@ __global__ void k_gather_moments(int64_t N, const int32_t *__restrict__ seg_ptr,
 
 void launch_gather(Ctx &c, const D4 *Xw_lab, const int32_t *seg_ptr, const int32_t *perm)
 {
+    join_assembly(c);  // and the gathered points
     int threads = 128;
     c.tbeg(PH_SEGMENTS);
     k_gather_moments<<<(unsigned)ceil_div(c.N, threads), threads, 0, c.stream>>>(

@@ -86,7 +86,9 @@ void launch_rk2(Ctx &c, int stage, double dt, const double *sol);
 void launch_assemble(Ctx &c, const D4 *x_lab, double *A64, float *A32, int64_t lda,
                      cudaStream_t s = nullptr, bool from_state = false);
 void launch_assemble32(Ctx &c, const D4 *x_lab, float *A32, int64_t lda);
-// make c.stream wait for the FP64 assembly running on the side stream, if any
+// make c.stream wait for the FP64 assembly running on the side stream, if any:
+// before its matrix is used, and before anything that it reads is written again
+// (the force points c.d_x, the segments, the gathered points)
 void join_assembly(Ctx &c);
 
 // ---- velocity at field points and tracers (velocity.cu) --------------------

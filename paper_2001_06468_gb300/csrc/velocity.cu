@@ -49,10 +49,12 @@ __device__ __noinline__ double2 inv_cube_fp64(double rho, double dg)
 
 // part[(s * P + p) * 3 + j] = sum over quadrature points q of range s of
 // S_jk w_q f_k(n(q)), q ascending in groups of VL_GROUP.  one = 1.0, nz = -0.0
-// (run-time values, so that a fused multiply-add stays one).
+// (run-time values, so that a fused multiply-add stays one).  N force points;
+// a quadrature point without a nearest one (no distance was finite: k_nearest
+// marks it -1) has no density, and the velocity is NaN.
 __global__ void __launch_bounds__(VL_THREADS)
     k_velocity_part(int64_t P, const D4 *__restrict__ xp, int64_t Q, const D4 *__restrict__ Xw,
-                    const int32_t *__restrict__ nn, const double *__restrict__ f, double eps2,
+                    const int32_t *__restrict__ nn, int64_t N, const double *__restrict__ f, double eps2,
                     int64_t q_per_split, double one, double nz, double *__restrict__ part)
 {
     __shared__ VelPoint sX[VL_CHUNK];
@@ -74,8 +76,11 @@ __global__ void __launch_bounds__(VL_THREADS)
         __syncthreads();
         for (int i = threadIdx.x; i < cnt; i += VL_THREADS) {
             const D4 X = Xw[c0 + i];
-            const double *fq = f + 3 * (int64_t)nn[c0 + i];
-            sX[i] = VelPoint{X.x, X.y, X.z, X.w * fq[0], X.w * fq[1], X.w * fq[2]};
+            const int64_t n = nn[c0 + i];
+            const bool has = n >= 0 && n < N;
+            const double *fq = f + (has ? 3 * n : 0);
+            const double w = has ? X.w : __longlong_as_double(0x7ff8000000000000LL);
+            sX[i] = VelPoint{X.x, X.y, X.z, w * fq[0], w * fq[1], w * fq[2]};
         }
         __syncthreads();
         if (idle) continue;
@@ -181,8 +186,8 @@ void launch_velocity(Ctx &c, const D4 *Xw, const D4 *xp, int64_t P, const double
     const int64_t qps = ceil_div(c.Q, splits);
     const double coef = 1.0 / (8.0 * kPi * c.mu);
     dim3 grid((unsigned)ceil_div(P, VL_THREADS), (unsigned)splits);
-    k_velocity_part<<<grid, VL_THREADS, 0, s>>>(P, xp, c.Q, Xw, c.d_nn, f, c.eps * c.eps, qps,
-                                                1.0, -0.0, part);
+    k_velocity_part<<<grid, VL_THREADS, 0, s>>>(P, xp, c.Q, Xw, c.d_nn, c.N, f, c.eps * c.eps,
+                                                qps, 1.0, -0.0, part);
     k_velocity_finish<<<(unsigned)ceil_div(3 * P, 128), 128, 0, s>>>(
         P, splits, part, coef, reinterpret_cast<double *>(u));
     c.launches += 2;

@@ -17,6 +17,7 @@
 #include <math.h>
 
 #include <algorithm>
+#include <cmath>
 
 #include "nrs_internal.cuh"
 
@@ -207,6 +208,12 @@ __device__ __forceinline__ void atomic_max_nonneg(double *p, double v)
               (unsigned long long)__double_as_longlong(v));
 }
 
+// |v| for a maximum norm: infinite if v is not a number (fmax would drop it)
+__device__ __forceinline__ double norm_term(double v)
+{
+    return isfinite(v) ? fabs(v) : __longlong_as_double(0x7ff0000000000000LL);
+}
+
 // part[s*n + i] = sum_{j in split s} A[i,j] v[j] for the FP64 matrix.  Each
 // thread owns two adjacent rows (one 16-byte load per column), so a warp reads
 // 512 contiguous bytes per column; rows i+1 >= n read the padding rows below n
@@ -235,7 +242,10 @@ __global__ void __launch_bounds__(MV_THREADS)
 // part[s*n + i] = sum_{j in split s} |A[i,j]|, laid out as k_gemv_part; `one` is
 // 1.0 (a fused multiply-add issues faster than an addition).  One more row of
 // blocks (blockIdx.y == splits) forms scal[SC_FXX] = ||x||_inf and scal[SC_BN]
-// = ||b||_inf and clears the maxima that the later kernels take by atomics.
+// = ||b||_inf and clears the maxima that the later kernels take by atomics.  The
+// norms of A and x, the exact residual's anchor, leave out what is not a number:
+// it poisons its own rows (fx_poison) and so the residual's norm, and the other
+// rows stay exact.
 __global__ void __launch_bounds__(MV_THREADS)
     k_rowsums_part(int64_t n, const double *__restrict__ A, int64_t lda, double one,
                    const double *__restrict__ x, const double *__restrict__ b,
@@ -366,9 +376,9 @@ __global__ void __launch_bounds__(MV_THREADS)
 }
 
 // out[i] = b[i] - (sum_s fx + sum_s part), the integer sums exact, rounded
-// once; *rn (zero before) = max |out[i]|.  A block takes 32 rows, its eight
-// warps the splits w, w + 8, ...: with one thread a row the chain of up to 64
-// dependent loads took 40 to 75 us.
+// once; *rn (zero before) = max |out[i]|, infinite if an out[i] is not finite.
+// A block takes 32 rows, its eight warps the splits w, w + 8, ...: with one thread
+// a row the chain of up to 64 dependent loads took 40 to 75 us.
 constexpr int FXF_WARPS = 8;
 __global__ void __launch_bounds__(32 * FXF_WARPS)
     k_gemv_finish_fx(int64_t n, const unsigned long long *__restrict__ fx,
@@ -402,7 +412,7 @@ __global__ void __launch_bounds__(32 * FXF_WARPS)
         r = fx_residual(b[i], S, fx_anchor(scal[SC_FXA], scal[SC_FXX]), es);
         out[i] = r;
     }
-    r = fmax(0.0, fabs(r));  // (not a number counts as nothing)
+    r = norm_term(r);
     for (int o = 16; o > 0; o >>= 1) r = fmax(r, __shfl_xor_sync(0xffffffffu, r, o));
     if (lane == 0) atomic_max_nonneg(rn, r);
 }
@@ -563,8 +573,8 @@ __global__ void __launch_bounds__(RED_THREADS)
 {
     double dn = 0.0, xn = 0.0;
     for (int64_t e = threadIdx.x; e < n; e += RED_THREADS) {
-        dn = fmax(dn, fabs(d[e]));
-        xn = fmax(xn, fabs(x[e]));
+        dn = fmax(dn, norm_term(d[e]));
+        xn = fmax(xn, norm_term(x[e]));
     }
     dn = block_max(dn);
     xn = block_max(xn);
@@ -573,7 +583,7 @@ __global__ void __launch_bounds__(RED_THREADS)
         scal[SC_XN] = xn;
         if (!isfinite(dn) || !isfinite(xn)) {
             atomicOr(status, ST_NONFINITE);
-            scal[SC_OUTER_DONE] = 1.0;
+            scal[SC_OUTER_DONE] = 2.0;  // done, but not converged
         } else if (dn <= tol * xn) {
             scal[SC_OUTER_DONE] = 1.0;
         } else if (scal[SC_DNPREV] > 0.0 && dn * (dn / scal[SC_DNPREV]) <= 1e-3 * tol * xn) {
@@ -588,12 +598,12 @@ __global__ void __launch_bounds__(RED_THREADS)
     }
 }
 
-// ||v||_inf into scal[slot]
+// ||v||_inf into scal[slot], infinite if an entry is not finite
 __global__ void __launch_bounds__(RED_THREADS)
     k_nrm_inf(int64_t n, const double *__restrict__ v, double *__restrict__ scal, int slot)
 {
     double m = 0.0;
-    for (int64_t e = threadIdx.x; e < n; e += RED_THREADS) m = fmax(m, fabs(v[e]));
+    for (int64_t e = threadIdx.x; e < n; e += RED_THREADS) m = fmax(m, norm_term(v[e]));
     m = block_max(m);
     if (threadIdx.x == 0) scal[slot] = m;
 }
@@ -851,7 +861,8 @@ nrs_status run_gmres_ir(Ctx &c, const double *b, double *x, const double *x0, nr
                 double sc[SC_COUNT];
                 CKE(cudaMemcpyAsync(sc, c.d_scal, sizeof(sc), cudaMemcpyDeviceToHost, c.stream));
                 CKE(cudaStreamSynchronize(c.stream));
-                if (sc[SC_RN] <= 1e-15 * (sc[SC_FXA] * sc[SC_XN] + sc[SC_BN])) {
+                if (std::isfinite(sc[SC_RN]) &&
+                    sc[SC_RN] <= 1e-15 * (sc[SC_FXA] * sc[SC_XN] + sc[SC_BN])) {
                     converged = true;
                     break;
                 }
@@ -901,7 +912,7 @@ nrs_status run_gmres_ir(Ctx &c, const double *b, double *x, const double *x0, nr
         double od = read_scalar(c, SC_OUTER_DONE, &e);
         if (e != cudaSuccess) CKE(e);
         if (od != 0.0) {
-            converged = true;
+            converged = od == 1.0;
             ++outer;
             break;
         }

@@ -106,10 +106,17 @@ void launch_kinematics(Ctx &c, const D4 *xi, const D4 *Xiw, const D4 *xidot, D4 
 // bounds.  The block stages the boxes that any of its warps kept, each warp
 // scans its own.  Points that are neighbours in index order are neighbours in
 // space on lattices and curves, so few boxes remain; for points in arbitrary
-// order all do, and the scan is the full one.  9200 force points and 92000
-// quadrature points of the channel, over all bodies: 893 us for the scan of
-// all pairs, 270 us with boxes kept for a whole block (those that straddle
-// two faces keep nearly all), 129 us kept by warps.
+// order all do: the scan is the full one, and what comes on top is a test of
+// every box a warp.  9200 force points and 92000 quadrature points of the
+// channel, over all bodies, map and segments with a cold L2: 970 us for the scan
+// of all pairs, 150 with boxes kept by warps (270 to 129 us of search when they
+// were kept for a whole block: those that straddle two faces keep nearly all).
+// Both clouds shuffled: 1029 and 1030 us, force points alone 987 and 1004,
+// quadrature points alone 1030 and 347; 9200 x 92000 random points 999 and 957;
+// 4000 x 32000 on 1728 lattice places (8 equally near force points on average) 513
+// and 353.  (Shuffled clouds took 1164 us when every point was asked whatever the
+// boxes looked like and a warp's kept boxes were looked up one by one, lattice
+// places 966 when more than four candidates a lane meant all force points again.)
 //
 // Two passes over the kept force points, staged through shared memory.
 // Pass 1 finds m_f, the smallest FP32 squared distance.  With C the largest
@@ -266,6 +273,17 @@ __global__ void __launch_bounds__(NN_THREADS)
             }
         }
     };
+    // the first cnt boxes of the tile in one run (a box at a time takes a tenth longer)
+    auto scan_all = [&](int cnt) {
+        if (active) {
+#pragma unroll 16
+            for (int i = sub; i < cnt * NN_BOX; i += NN_SPLIT) {
+                const float4 v = tile[i];
+                const float dx = v.x - fx, dy = v.y - fy, dz = v.z - fz;
+                best = fminf(best, dx * dx + dy * dy + dz * dz);
+            }
+        }
+    };
     // the squared bound above for the smallest distance so far, and 1e-43 for the
     // absolute rounding of squares that are subnormal (distances below 1e-19)
     auto bound = [&]() {
@@ -314,6 +332,26 @@ __global__ void __launch_bounds__(NN_THREADS)
         }
     };
     constexpr int NN_MANY = 16;  // kept boxes of a chunk from which on each point is asked
+    // whether asking can leave boxes out: not if half of those kept hold the warp's
+    // first point (force points in no spatial order: every box is the whole cloud)
+    auto worth_asking = [&](int64_t k0, int words, unsigned mine) {
+        const float px = __shfl_sync(0xffffffffu, fx, 0), py = __shfl_sync(0xffffffffu, fy, 0);
+        const float pz = __shfl_sync(0xffffffffu, fz, 0);
+        int all = 0, hold = 0;
+        for (int w = 0; w < words; ++w) {
+            const unsigned bits = __shfl_sync(0xffffffffu, mine, w);
+            if (!bits) continue;
+            bool in = (bits >> lane) & 1u;
+            if (in) {
+                const int64_t k = k0 + 32 * w + lane;
+                const float4 l = boxes[2 * k], h = boxes[2 * k + 1];
+                in = l.x <= px && px <= h.x && l.y <= py && py <= h.y && l.z <= pz && pz <= h.z;
+            }
+            hold += __popc(__ballot_sync(0xffffffffu, in));
+            all += __popc(bits);
+        }
+        return 2 * hold < all;
+    };
     bool seeded = false;
     // keeps, of the chunk of NN_THREADS boxes from k0 on, those within th of one
     // of the warp's points; returns how many some warp of the block kept
@@ -334,7 +372,8 @@ __global__ void __launch_bounds__(NN_THREADS)
             const unsigned bal = __ballot_sync(0xffffffffu, in);
             if (lane == w) mine = bal;
         }
-        if (__reduce_add_sync(0xffffffffu, __popc(mine)) > NN_MANY) {
+        if (__reduce_add_sync(0xffffffffu, __popc(mine)) > NN_MANY &&
+            worth_asking(k0, words, mine)) {
             // (in the first chunk, where no other warp looks at this one's slice of
             // the tile)
             if (!seeded && k0 == b_lo) {
@@ -382,7 +421,11 @@ __global__ void __launch_bounds__(NN_THREADS)
         __syncthreads();
         return total;
     };
-    auto kept_by_me = [&](int r) { return (mask[warp][r >> 5] >> (r & 31)) & 1u; };
+    // which of the cnt staged boxes list[j], ... this warp kept
+    auto mine_of = [&](int j, int cnt) {
+        const int r = lane < cnt ? list[j + lane] : 0;
+        return __ballot_sync(0xffffffffu, lane < cnt && ((mask[warp][r >> 5] >> (r & 31)) & 1u));
+    };
 
     if (b_hi > b_lo) {
         stage(seed);
@@ -399,39 +442,60 @@ __global__ void __launch_bounds__(NN_THREADS)
             const int cnt = min(NN_BOXES, kept - j);
             if (warp < cnt) stage(k0 + list[j + warp]);
             __syncthreads();
-            for (int s = 0; s < cnt; ++s)
-                if (kept_by_me(list[j + s])) scan(s);
+            const unsigned todo = mine_of(j, cnt);
+            if (todo == (1u << cnt) - 1u) {
+                scan_all(cnt);
+            } else {
+                for (unsigned m = todo; m; m &= m - 1) scan(__ffs(m) - 1);
+            }
         }
         if (!one_chunk) th = bound();
     }
     __syncthreads();  // s_cmax is final
     th = bound();
 
-    // this lane's candidates: how many, and the first four (from n_lo on)
+    double best64 = __longlong_as_double(0x7ff0000000000000LL);
+    int64_t arg = -1;
+    // (the candidates do not come in ascending order: the lowest index of equal ones)
+    auto try64 = [&](int64_t n) {
+        const D4 p = x[n];
+        double ex = __dsub_rn(p.x, qx), ey = __dsub_rn(p.y, qy), ez = __dsub_rn(p.z, qz);
+        double s = __dadd_rn(__dadd_rn(__dmul_rn(ex, ex), __dmul_rn(ey, ey)), __dmul_rn(ez, ez));
+        if (s < best64 || (s == best64 && n < arg)) {
+            best64 = s;
+            arg = n;
+        }
+    };
+    // this lane's candidates: how many, and the first four (from n_lo on); more, of
+    // force points at nearly the same distance, are decided at once
     int found = 0;
     int32_t cand[4] = {0, 0, 0, 0};
     auto decide = [&](int slot, int64_t k) {
         if (active) {
+            unsigned near = 0u;
 #pragma unroll
-            for (int i = sub; i < NN_BOX; i += NN_SPLIT) {
-                const float4 v = tile[slot * NN_BOX + i];
+            for (int u = 0; u < NN_BOX / NN_SPLIT; ++u) {
+                const float4 v = tile[slot * NN_BOX + sub + NN_SPLIT * u];
                 const float dx = v.x - fx, dy = v.y - fy, dz = v.z - fz;
-                const float d2 = dx * dx + dy * dy + dz * dz;
-                if (d2 <= th) {
-                    const int32_t n = (int32_t)(k * NN_BOX + i - n_lo);
-                    if (found == 0) cand[0] = n;
-                    if (found == 1) cand[1] = n;
-                    if (found == 2) cand[2] = n;
-                    if (found == 3) cand[3] = n;
-                    ++found;
-                }
+                if (dx * dx + dy * dy + dz * dz <= th) near |= 1u << u;
+            }
+            for (; near; near &= near - 1u) {
+                const int32_t n = (int32_t)(k * NN_BOX + sub + NN_SPLIT * (__ffs(near) - 1) - n_lo);
+                if (found == 0) cand[0] = n;
+                if (found == 1) cand[1] = n;
+                if (found == 2) cand[2] = n;
+                if (found == 3) cand[3] = n;
+                if (found > 3) try64(n_lo + n);
+                ++found;
             }
         }
     };
     if (one_chunk && kept <= NN_BOXES) {
         // the tile still holds them all
-        for (int s = 0; s < kept; ++s)
-            if (kept_by_me(list[s])) decide(s, b_lo + list[s]);
+        for (unsigned m = mine_of(0, kept); m; m &= m - 1) {
+            const int s = __ffs(m) - 1;
+            decide(s, b_lo + list[s]);
+        }
     } else {
         seeded = true;  // every distance is known: th stays
         for (int64_t k0 = b_lo; k0 < b_hi; k0 += NN_THREADS) {
@@ -441,47 +505,27 @@ __global__ void __launch_bounds__(NN_THREADS)
                 const int cnt = min(NN_BOXES, kept - j);
                 if (warp < cnt) stage(k0 + list[j + warp]);
                 __syncthreads();
-                for (int s = 0; s < cnt; ++s)
-                    if (kept_by_me(list[j + s])) decide(s, k0 + list[j + s]);
+                for (unsigned m = mine_of(j, cnt); m; m &= m - 1) {
+                    const int s = __ffs(m) - 1;
+                    decide(s, k0 + list[j + s]);
+                }
             }
         }
     }
     // One candidate in all, at a finite distance, is the neighbour; more are
     // decided in FP64 (76 clocks of the pipe an operation: only then).
-    int total = found, most = found;
+    int total = found;
 #pragma unroll
-    for (int o = 1; o < NN_SPLIT; o <<= 1) {
-        total += __shfl_xor_sync(0xffffffffu, total, o);
-        most = max(most, __shfl_xor_sync(0xffffffffu, most, o));
-    }
-    double best64 = __longlong_as_double(0x7ff0000000000000LL);
-    int64_t arg = -1;
-    auto try64 = [&](int64_t n) {
-        const D4 p = x[n];
-        double ex = __dsub_rn(p.x, qx), ey = __dsub_rn(p.y, qy), ez = __dsub_rn(p.z, qz);
-        double s = __dadd_rn(__dadd_rn(__dmul_rn(ex, ex), __dmul_rn(ey, ey)), __dmul_rn(ez, ez));
-        if (s < best64) {
-            best64 = s;
-            arg = n;
-        }
-    };
+    for (int o = 1; o < NN_SPLIT; o <<= 1) total += __shfl_xor_sync(0xffffffffu, total, o);
     if (total == 1 && best < inf) {
         if (found) {
             arg = n_lo + cand[0];
             best64 = 0.0;
         }
-    } else if (most <= 4) {
+    } else {
 #pragma unroll
         for (int c = 0; c < 4; ++c)
             if (c < found) try64(n_lo + cand[c]);
-    } else {
-        // many at nearly the same distance: every force point again
-        for (int64_t n = n_lo + sub; n < n_hi; n += NN_SPLIT) {
-            const D4 p = x[n];
-            const float dx = nearest_float(p.x) - fx, dy = nearest_float(p.y) - fy;
-            const float dz = nearest_float(p.z) - fz;
-            if (dx * dx + dy * dy + dz * dz <= th) try64(n);
-        }
     }
 #pragma unroll
     for (int o = 1; o < NN_SPLIT; o <<= 1) {

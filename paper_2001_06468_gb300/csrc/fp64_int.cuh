@@ -21,13 +21,13 @@
 // the exponents.  The functions compile for the host too (the CPU test).
 #pragma once
 
+#include <math.h>
 #include <stdint.h>
 #include <string.h>
 
 #ifdef __CUDACC__
 #define NRS_HD __host__ __device__ __forceinline__
 #else
-#include <math.h>
 #define NRS_HD inline
 #endif
 
@@ -233,6 +233,17 @@ NRS_HD Sig inv_rho_sqrt(double rho_d, bool &tie)
     // with it may meet another factor of 2^53
     const uint32_t carry = hi32(s) >> 21;
     return Sig{s - ((uint64_t)carry << 52), (2045u << 20) - p.f + (carry << 20)};
+}
+
+// 1/x from y within 2^-19 of it (relative): one step of the hyperpower iteration
+// of order three, y (1 + e + e^2) with e = 1 - x y (Altman, "An optimum cubically
+// convergent iterative method of inverting a linear bounded operator in Hilbert
+// space", 1960).  The step leaves e^3, and its last operation rounds once: within
+// 0.57 units in the last place.
+NRS_HD double rcp_refined(double x, double y)
+{
+    const double e = fma(-x, y, 1.0);
+    return fma(y, fma(e, e, e), y);
 }
 
 // v = hi + lo as two floats: hi the nearest float (a tie away from zero), lo

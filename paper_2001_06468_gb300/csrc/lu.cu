@@ -38,14 +38,13 @@ constexpr int LU_DIAG_SMEM = (LU_NB * LU_LD + 4 * LU_HB * (LU_HB + 1)) * (int)si
 
 constexpr int DF_ROWS = 5;  // rows a warp updates at once
 
-// 1/x to about one unit in the last place: a seed of 20 bits and one cubic
-// Newton step, y (1 + e + e^2) with e = 1 - x y
+// 1/x within one unit in the last place (rcp_refined): the seed instruction gives
+// 20 bits
 __device__ __forceinline__ double lu_rcp(double x)
 {
     double y;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-    const double e = fma(-x, y, 1.0);
-    return fma(y, fma(e, e, e), y);
+    return rcp_refined(x, y);
 }
 
 // what its launch asks for: no other CTA of the factorisation fits beside it

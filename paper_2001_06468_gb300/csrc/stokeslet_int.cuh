@@ -26,13 +26,22 @@ struct FmaOps {
     NRS_HD double mul(double a, double b) const { return fma(a, b, nz); }
 };
 
+// Components of r below the first count as zero in terms_int; from the second
+// on, infinities and NaN among them, the pair is left to the general path
+// (rho leaves the integer path's range there, but a square formed from wrapped
+// exponents need not).
+constexpr uint32_t kTinyHi = 873u << 20;  // 2^-150
+constexpr uint32_t kFarHi = 1073u << 20;  // 2^50
+
 // A quadrature point staged for the pair loop: its weight also as a
 // significand for the integer products (shifted left by one, sign and
-// exponent field), usable when `ok`.
+// exponent field), and the high word from which a component of r sends the pair
+// to the general path: kFarHi, or zero (every pair) if the weight is outside the
+// integer path's range.
 struct alignas(16) StagedX {
     double x, y, z, w;
     uint64_t w2;
-    uint32_t wf, ok;
+    uint32_t wf, far_hi;
 };
 
 NRS_HD StagedX stage_weighted(double x, double y, double z, double w)
@@ -47,16 +56,9 @@ NRS_HD StagedX stage_weighted(double x, double y, double z, double w)
     v.wf = sw.f;
     // 2^-200 <= |w| < 2^200 (zero, subnormal and non-finite weights excluded)
     const uint32_t ex = (sw.f >> 20) & 0x7ffu;
-    v.ok = ex - 823u < 400u;
+    v.far_hi = ex - 823u < 400u ? kFarHi : 0u;
     return v;
 }
-
-// Components of r below the first count as zero in terms_int; from the second
-// on, infinities and NaN among them, the pair is left to the general path
-// (rho leaves the integer path's range there, but a square formed from wrapped
-// exponents need not).
-constexpr uint32_t kTinyHi = 873u << 20;  // 2^-150
-constexpr uint32_t kFarHi = 1073u << 20;  // 2^50
 
 NRS_HD uint32_t magnitude_hi(double r) { return hi32(double_bits(r)) & 0x7fffffffu; }
 NRS_HD bool tiny(double r) { return magnitude_hi(r) < kTinyHi; }
@@ -67,7 +69,9 @@ NRS_HD bool tiny(double r) { return magnitude_hi(r) < kTinyHi; }
 // pipe, rounded identically (fp64_int.cuh).  A component of r below 2^-150 is
 // taken as zero (then a product with it is a zero, whose sign does not matter:
 // a sum starts at +0).  odd = 1: some component was; 2 and more: the general
-// path is needed.
+// path is needed.  (The components' range and the weight's in one comparison:
+// 2000 x 20000 points 1748 us, 1737 without the components'; in two, 1781, with
+// spills.)
 NRS_HD Acc6 terms_int(double mx, double my, double mz, const StagedX &X, double eps2, double two_e2,
                       const FmaOps &op, int &odd)
 {
@@ -76,7 +80,7 @@ NRS_HD Acc6 terms_int(double mx, double my, double mz, const StagedX &X, double 
     const bool tx = hx < kTinyHi, ty = hy < kTinyHi, tz = hz < kTinyHi;
     const Sig ux = unpack(rx), uy = unpack(ry), uz = unpack(rz);
     const uint32_t hxy = hx > hy ? hx : hy;
-    bool bad = !X.ok || (hxy > hz ? hxy : hz) >= kFarHi;
+    bool bad = (hxy > hz ? hxy : hz) >= X.far_hi;
     const Sig pxx = mul_sig(ux, ux.m << 1, ux.f, bad);
     const Sig pyy = mul_sig(uy, uy.m << 1, uy.f, bad);
     const Sig pzz = mul_sig(uz, uz.m << 1, uz.f, bad);

@@ -264,6 +264,7 @@ nrs_status do_segments_and_assemble(Ctx *c, const D4 *x_lab, const D4 *Xw_lab, b
             nrs::launch_assemble(*c, x_lab, c->d_A64, nullptr, c->lda, c->stream3, from_state);
             CK(cudaEventRecord(c->ev_asm_done, c->stream3));
             c->asm_pending = true;
+            c->asm_captured = nrs::is_capturing(c->stream);
         }
     } else {
         // one FP64 pass; with an FP32 copy, that copy is the rounded FP64 entries
@@ -326,10 +327,26 @@ nrs_status mlp_alloc(Ctx *c)
 
 namespace nrs {
 
+bool is_capturing(cudaStream_t s)
+{
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    // (the legacy stream during another stream's capture: an error, and not capturing)
+    if (cudaStreamIsCapturing(s, &st) != cudaSuccess) cudaGetLastError();
+    return st == cudaStreamCaptureStatusActive;
+}
+
 void join_assembly(Ctx &c)
 {
     if (!c.asm_pending) return;
-    cudaStreamWaitEvent(c.stream, c.ev_asm_done, 0);
+    if (!c.asm_captured && is_capturing(c.stream)) {
+        // a capture cannot wait for work from before it: the host does
+        cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+        cudaThreadExchangeStreamCaptureMode(&mode);
+        cudaEventSynchronize(c.ev_asm_done);
+        cudaThreadExchangeStreamCaptureMode(&mode);
+    } else {
+        cudaStreamWaitEvent(c.stream, c.ev_asm_done, 0);
+    }
     c.asm_pending = false;
 }
 

@@ -90,6 +90,7 @@ void launch_assemble32(Ctx &c, const D4 *x_lab, float *A32, int64_t lda);
 // before its matrix is used, and before anything that it reads is written again
 // (the force points c.d_x, the segments, the gathered points)
 void join_assembly(Ctx &c);
+bool is_capturing(cudaStream_t s);
 
 // ---- velocity at field points and tracers (velocity.cu) --------------------
 int velocity_splits(const Ctx &c, int64_t P);
@@ -172,6 +173,7 @@ struct Ctx {
     cudaStream_t stream3 = nullptr;              // FP64 assembly overlapping the factorisation
     cudaEvent_t ev_asm = nullptr, ev_asm_done = nullptr;
     bool asm_pending = false;                    // stream3 holds an FP64 assembly not yet joined
+    bool asm_captured = false;                   //   recorded in a capture of the caller's stream
     int lo_eval = 0;  // FP32 copy for the factor: 0 evaluated in FP32 (overlapped), 1 rounded FP64
     int asm_side_ctas = 3;  // CTAs per SM of the FP64 assembly beside the factorisation
     unsigned int *d_asm_claim = nullptr;  // its tile counter there

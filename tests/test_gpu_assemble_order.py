@@ -73,3 +73,23 @@ def test_a_recorded_step_after_an_assembly(nrs, recorded):
             ctx.step(s0, sh, 0.01, sol=sol)
         got.append(sol.cpu().numpy())
     assert np.array_equal(got[0], got[1])
+
+
+def test_a_map_captured_after_an_assembly(nrs):
+    # the capture of a call that rewrites the segments, with an assembly from
+    # before it still unjoined
+    (x0, X0), (x1, X1) = _cloud(34), _cloud(35)
+    N, Q = x0.shape[0], X0.shape[0]
+    stream = torch.cuda.Stream()
+    ctx = nrs.Context([0, N], [0, Q], [nrs.PRESCRIBED], eps=0.05, factor_prec="tf32", stream=stream)
+    with torch.cuda.stream(stream):
+        want = [t.cpu() for t in ctx.nearest_build(x1, X1)]
+        ctx.nearest_build(x0, X0)
+        ctx.assemble(x0, X0, want_matrix=False)
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=stream):
+        got = ctx.nearest_build(x1, X1)
+    graph.replay()
+    torch.cuda.synchronize()
+    for a, b in zip(got, want):
+        assert torch.equal(a.cpu(), b)

@@ -87,11 +87,12 @@ TF32_OVER_BF16 = 1.1 / 2.25      # nominal dense TF32 / BF16 tensor throughput
 SM_COUNT_NOMINAL = 152
 FP32_LANES_PER_SM = 128
 PAIR_INSTR = 20                  # FP32-pipe instructions per (force, quadrature) pair
-# Work counted in FP64 operations, most of which the kernels do on the integer
-# pipe (correctly rounded, or exactly): a fraction of the FP64 pipe's rate above 1
-# means that much more than that pipe alone could do
+# Work counted in the FP64 operations that the plain form of a kernel takes.  The
+# kernels do most of it on the integer pipe: a fraction of the FP64 pipe's rate is
+# then no utilisation of that pipe, and above 1 it is more than that pipe alone
+# could do
 ASM64_OPS_PER_PAIR = 40          # per pair of the bit-exact assembly
-RES_OPS_PER_ENTRY = 3            # per matrix entry of the extended residual
+RES_OPS_PER_ENTRY = 3            # per matrix entry of the extended residual, which issues none
 TOL = 1e-10
 
 
@@ -217,10 +218,10 @@ NCU_TRAFFIC = {
                      "sha1": "", "scale": None},
     # one solve at n = 13824 (cold start, 2 refinement steps -- the first on a
     # working-precision residual, the second on the exact one -- and 4 GMRES
-    # iterations; the three-CTAs-per-SM variant on 456 CTAs): 16.101 + 0.056 GB
+    # iterations; the three-CTAs-per-SM variant on 456 CTAs): 16.102 + 0.053 GB
     # against 7 passes over A (8 n^2) and M (4 n^2) = 16.05 GB
-    "k_gmres_ir": {"bytes": None, "ratio": (16100587008 + 56127744) / (12.0 * 13824 ** 2 * 7),
-                   "file": "paper_2001_06468_gb300/csrc/gmres_persistent.cu", "sha1": "0a46b9864734",
+    "k_gmres_ir": {"bytes": None, "ratio": (16101891584 + 53305088) / (12.0 * 13824 ** 2 * 7),
+                   "file": "paper_2001_06468_gb300/csrc/gmres_persistent.cu", "sha1": "ac89669e4a72",
                    "scale": "traffic / algorithmic bytes at n = 13824, times the record's bytes"},
 }
 
@@ -355,11 +356,13 @@ def rooflines(ph_ms, ph_spans, n, pairs, peaks, peak_src, sm_mhz, solve_stats, p
                   products, exact from A in FP64 or in working precision from its
                   float-pair copy, and the GMRES products: 8 bytes an entry each)
                   + (outer + inner + 1) 4 n^2 bytes of M; + 8 n^2 (||A||_inf, once
-                  per launch); exact x 3 n^2 (extended residual: product, its error
-                  and the error sum, all on the integer pipe) + n^2
-                  (||A||_inf) + (inner + working) x n^2 (the GMRES and residual
-                  products, when in FP64) FP64 operations.  Without the residual
-                  counts, every refinement step counts one exact residual."""
+                  per launch).  fp64_gops counts exact x 3 n^2 (the extended
+                  residual as rounded products, their errors and the errors' sum;
+                  the kernel forms 106-bit products and 192-bit sums on the integer
+                  pipe instead) + n^2 (||A||_inf) + (inner + working) x n^2 (the
+                  GMRES and residual products, when in FP64); fp64_issued_gops leaves
+                  the extended residual out.  Without the residual counts, every
+                  refinement step counts one exact residual."""
     P = derived_peaks(peaks, sm_mhz)
 
     def per_launch(ph):
@@ -468,16 +471,19 @@ def rooflines(ph_ms, ph_spans, n, pairs, peaks, peak_src, sm_mhz, solve_stats, p
         wk = solve_stats.get("working_mean", 0.0)
         t = per_launch("krylov")
         b = 8.0 * n * n * (ex + wk + i + 1) + 4.0 * n * n * (o + i + 1)
-        # FP64 operations: the exact residuals, the ||A||_inf pass, and the
-        # GMRES and working-precision residual products unless they run on the
-        # float-pair copy (FP32 pipe)
-        ops = RES_OPS_PER_ENTRY * n * n * ex + n * n * (1 + (0 if arnoldi_df else i + wk))
+        # FP64 operations: the ||A||_inf pass, and the GMRES and working-precision
+        # residual products unless they run on the float-pair copy (FP32 pipe); the
+        # exact residuals (integer pipe) are counted on top
+        issued = n * n * (1 + (0 if arnoldi_df else i + wk))
+        ops = RES_OPS_PER_ENTRY * n * n * ex + issued
         recs["krylov"] = {
             "kernel": "k_gmres_ir (persistent GMRES-IR, one cooperative launch per solve)",
             "bound": "hbm", "achieved": b / t / 1e9, "peak": P["hbm_gbs"], "unit": "GB/s",
             "frac": b / t / 1e9 / P["hbm_gbs"], "peak_source": peak_src + " HBM copy",
             "work_per_launch": b, "work_unit": "bytes of A (FP64) and M (FP32) streamed",
             "fp64_gops": ops / t / 1e9, "fp64_frac": ops / t / 1e9 / P["fp64_gops"],
+            "fp64_issued_gops": issued / t / 1e9,
+            "fp64_issued_frac": issued / t / 1e9 / P["fp64_gops"],
             "outer_mean": o, "inner_mean": i, "ms_per_launch": t * 1e3,
             "launches": ph_spans["krylov"], "traffic": _traffic("k_gmres_ir", n, b)}
     return recs

@@ -160,7 +160,8 @@ typedef struct {
     int32_t inner;          /* total GMRES iterations                         */
     int32_t converged;      /* 1 if the tolerance was met                     */
     int32_t status;         /* nrs_status of the device status word           */
-    double backward_err;    /* ||b - A x||_inf / (||A||_inf ||x||_inf + ||b||_inf) */
+    double backward_err;    /* ||b - A x||_inf / (||A||_inf ||x||_inf + ||b||_inf); not
+                               finite if the residual is not                  */
     double last_update;     /* ||dx||_inf / ||x||_inf of the last step         */
 } nrs_solve_report;
 
@@ -394,8 +395,10 @@ nrs_status nrs_residual_counters(const nrs_ctx *ctx, int64_t *exact, int64_t *wo
  *   u [P*4]   device output (u_x, u_y, u_z, 0)
  * n(q) is the nearest-neighbour map of the last nrs_nearest_build or
  * nrs_step.  NRS_EINVAL before there is one (or, with Xw NULL, before the
- * first nrs_step).  The first call with a larger P allocates the partial-sum
- * workspace (synchronises). */
+ * first nrs_step).  A quadrature point without a nearest force point (the map
+ * says -1: no distance was finite) has no density: every velocity is NaN.  The
+ * first call with a larger P allocates the partial-sum workspace
+ * (synchronises). */
 nrs_status nrs_velocity(nrs_ctx *ctx, const double *Xw, const double *xp, int64_t P, const double *f,
                         double *u);
 

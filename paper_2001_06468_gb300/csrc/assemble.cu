@@ -36,7 +36,7 @@ constexpr int AS_CHUNK = 512;
 // does not depend on the chunk)
 constexpr int AS64_CHUNK = 128;
 // order from which the FP64 assembly beside a lone factorisation takes the
-// integer form
+// integer form (launch_assemble: both sides)
 constexpr int64_t ASM_INT_MIN_N = 4096;
 
 __device__ __forceinline__ StagedX stage_point(const D4 &p)
@@ -485,10 +485,15 @@ void launch_assemble(Ctx &c, const D4 *x_lab, double *A64, float *A32, int64_t l
         // the assembly either way, and its chain of latency-bound kernels suffers
         // more from the integer form's issue slots and registers than from the
         // FP64 form's longer run (single swimmer's step: 3.18 ms with the FP64
-        // form, 3.27 with the integer one); among the chains of a batch (32
-        // reduced nodes: 37.1 and 25.2 ms), beside the two-level updates and beside
-        // one-level updates that take longer than the chain (n = 5115: the
-        // assembly alone 2.6 and 1.2 ms) the integer form is the better one.
+        // form, 3.27 with the integer one; assembly and factorisation at n = 2424
+        // 1.28 and 1.42 ms, n = 3633 2.31 and 2.48).  Among the chains of a batch
+        // (32 reduced nodes: 37.1 and 25.2 ms) and beside the two-level updates the
+        // integer form is the better one.  In between neither is: with 8 quadrature
+        // points a force point the FP64 form stays 4 to 6 % ahead (n = 4140 3.16 and
+        // 3.37 ms, 5115 5.60 and 5.96, 7221 12.6 and 13.2, 8001 18.5 and 16.7), with
+        // 16 its long CTAs can hold the SMs that the chain waits for (n = 5115 10.3
+        // to 10.9 and 6.18 ms, 6012 14.4 to 15.3 and 9.04).  The line is where an
+        // assembly is long enough for that loss to outweigh the gain.
         if (!c.pg_shared && c.n < ASM_INT_MIN_N) kernel = k_assemble64<false>;
         grid = std::min<int64_t>(tiles, (int64_t)c.asm_side_ctas * c.num_sms);
     }

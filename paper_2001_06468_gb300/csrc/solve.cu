@@ -717,9 +717,12 @@ static void residual(Ctx &c, const double *x, const double *b, double *r)
         return;
     }
     // two blocks an SM, as the plain products; six where the matrix comes from HBM
-    // (n = 5115: 229 us with two, 113 with six, the mixed solve 6408 and 6302 us;
-    // n = 2592, from L2: six solves with reports 4004 and 4051 us, the sums of
-    // more splits taking longer).  The sums are exact however they are split.
+    // (this product at n = 5115: 229 us with two, 113 with six, the mixed solve 6408
+    // and 6302 us; n = 2592, from L2: six solves with reports 4004 and 4051 us, the
+    // sums of more splits taking longer).  The line is on the safe side: nrs_residual
+    // and one solve with its report at n = 2736 106 and 568 us with two, 91 and 568
+    // with six, at n = 3945 226 and 1152, 157 and 1083.  The sums are exact however
+    // they are split.
     const int64_t rowblocks = ceil_div(c.n, 2 * MV_THREADS);
     const int64_t blocks = (c.n < FX_HBM_N ? 2 : 6) * (int64_t)c.num_sms;
     const int splits = (int)std::min<int64_t>(std::min<int64_t>(64, c.n), ceil_div(blocks, rowblocks));
